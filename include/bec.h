@@ -406,7 +406,9 @@ bec_status bec_inject_fault(int kind);
  * caches the choice for the process per (precision, dim, nx, N); force = 1
  * re-times a cached shape.  The width only regroups lines, so every choice
  * gives the same result bit for bit.  Transforms shorter than 32 and the
- * multigrid and learned routes have nothing to tune (the report is zero).
+ * multigrid and learned routes have nothing to tune (the report is zero);
+ * FP64 problems with both transforms of length >= 32 run fixed-point passes
+ * of a fixed width (the times stay 0).
  * bec_batch_create tunes each instance.  When the environment variable
  * BEC_TUNE_CACHE names a file, choices are also read from and appended to
  * it, so that later processes skip the timing.  Synchronises. */

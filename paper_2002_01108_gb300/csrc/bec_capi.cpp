@@ -99,6 +99,7 @@ void free_all(bec_problem* p) {
   destroy_profiler(p);
   net_free(p);
   mg_free(p);
+  fx_free(p);
   for (auto& g : p->graphs)
     if (g.exec) cudaGraphExecDestroy(g.exec);
   p->graphs.clear();
@@ -273,8 +274,6 @@ bec_status bec_allocate_problem(const bec_problem_desc* d, void* stream, bec_pro
   chain(dmalloc(&t.eis32, N));
   chain(dmalloc(&t.lamf64, N / 2 + 1));
   chain(dmalloc(&t.lamf32, N / 2 + 1));
-  if (d->precision == BEC_PC_FP64 && d->route == BEC_ROUTE_FST)
-    chain(dmalloc(&t.rinv64, (size_t)p->J * (N / 2 + 1)));
   if (mgroute && s == BEC_OK) {
     p->mg.pre = d->mg_pre == 0 ? 1 : d->mg_pre;
     p->mg.post = (d->mg_pre == 0 && d->mg_post == 0) ? 1 : d->mg_post;
@@ -349,6 +348,12 @@ bec_status bec_allocate_problem(const bec_problem_desc* d, void* stream, bec_pro
       s = BEC_ENOMEM;
     }
   }
+  // The fixed-point route's table takes twice the floating-point route's, so it
+  // comes after everything else: where it does not fit, the problem runs the
+  // floating-point passes as before.
+  if (s == BEC_OK && d->precision == BEC_PC_FP64 && d->route == BEC_ROUTE_FST &&
+      (!fx_wanted(d, t.space.logn, t.time.logn) || fx_setup(p) != BEC_OK))
+    chain(dmalloc(&t.rinv64, (size_t)p->J * (N / 2 + 1)));
   if (s != BEC_OK) {
     free_all(p);
     delete p;
@@ -457,6 +462,7 @@ bec_status bec_set_eps(bec_problem* p, double eps) {
   BEC_TRY(upload(t.lamf64, lam, p->stream));
   BEC_TRY(upload(t.lamf32, lam32, p->stream));
   if (t.rinv64) BEC_TRY(launch_rinv_table(p));
+  if (fx_applies(p)) BEC_TRY(fx_set_eps(p, es));
   if (p->mg.ilu) BEC_TRY(mg_ilu_setup(p));
   BEC_CUDA_TRY(cudaStreamSynchronize(p->stream));
   p->eps = eps;

@@ -32,6 +32,14 @@ bec_status enqueue_scalar_read(bec_problem* p) {
 }  // namespace
 
 // z = P_eps^{-1} (s y), s = *scale_dev (1 if null)
+double pinv_scale(const bec_problem* p) {
+  const double n = (double)(p->m + 1);
+  const double per_axis = (2.0 / n) / 16.0;   // (orthonormal / raw)^2 for one forward+inverse pair
+  double scale = 0.5 / p->N;
+  for (int d = 0; d < p->dim; ++d) scale *= per_axis;
+  return scale;
+}
+
 bec_status apply_pinv(bec_problem* p, const double* y, double* z, const double* scale_dev) {
   NvtxRange range("bec P_eps^-1");
   const int fp64 = p->desc.precision == BEC_PC_FP64;
@@ -46,10 +54,14 @@ bec_status apply_pinv(bec_problem* p, const double* y, double* z, const double* 
     if (learned && !net_rejected(p)) BEC_TRY(net_correct(p));
     return launch_time_inv(p, p->mg.lv[0].x, z, fp64);
   }
-  const double n = (double)(p->m + 1);
-  const double per_axis = (2.0 / n) / 16.0;   // (orthonormal / raw)^2 for one forward+inverse pair
-  double scale = 0.5 / p->N;
-  for (int d = 0; d < p->dim; ++d) scale *= per_axis;
+  if (fx_applies(p)) {
+    BEC_TRY(launch_fx_rows(p, y, z, true));
+    if (p->dim >= 2) BEC_TRY(launch_fx_cols(p, z, true));
+    BEC_TRY(launch_fx_time(p, z, scale_dev));
+    if (p->dim >= 2) BEC_TRY(launch_fx_cols(p, z, false));
+    return launch_fx_rows(p, z, z, false);
+  }
+  const double scale = pinv_scale(p);
   const long long rows = p->J / p->m * p->N;    // lines along x
   if (fp64) {
     BEC_TRY(launch_dst_rows(p, y, 1, z, 1, rows, 1));

@@ -60,6 +60,24 @@ struct PcTables {
   double* rinv64 = nullptr;
 };
 
+// Fixed-point route of the FP64 sine-transform P_eps^{-1} (bec_fx.cuh); all
+// null when the problem runs the floating-point passes.
+struct FxTables {
+  void* tables = nullptr;    // the allocation that holds all but q
+  void* tw_space = nullptr;  // scaled twiddles of n = nx + 1 and of N
+  void* tw_time = nullptr;
+  void* sinw = nullptr;      // 2 sin(j pi / n) - 1
+  void* q = nullptr;         // [N/2+1][J] complex: scale / (lambda'_k + tau mu_q), per mode 2^-qe
+  int lpb = 0;               // line pairs a block transforms
+  int* qe = nullptr;         // exponents of q, one a tile of 2 lpb modes
+  int* e0 = nullptr;         // exponents of the tiles between the passes
+  int* e1 = nullptr;
+  int* em = nullptr;         // exponents of the time pass's tiles
+  int* xadd = nullptr;       // [N] exponents of eps^{-j/N} times the apply's scale
+  void* esm = nullptr;       // [N] eps^{j/N}: mantissas and exponents
+  int* ese = nullptr;
+};
+
 // Event pairs around kernel launches (bec_profile_start / bec_profile_stop).
 struct Profiler {
   bool on = false;
@@ -116,6 +134,7 @@ struct bec_problem {
   long long launches = 0;
 
   bec::PcTables tab;
+  bec::FxTables fx;
   bec::TileChoice tile;         // block widths of the P_eps^{-1} passes
   void* pc_scratch = nullptr;   // N x Jp elements of the preconditioner's type
   // Row length and points per time slice of pc_scratch: in FP32 every row
@@ -195,6 +214,9 @@ bec_status gmres_run_result(const GmresRun& r);
 bec_status gmres_solve_one(bec_problem* p, const double* f, double* u,
                            const bec_gmres_opts* o, bec_gmres_info* info);
 bec_status check_gmres_opts(const bec_problem* p, const bec_gmres_opts* o);
+// normalisation of the transforms of P_eps^{-1}: the raw forward and inverse
+// sine transforms give (8 n)^dim times their argument, the FFT pair 2 N times
+double pinv_scale(const bec_problem* p);
 // z = P_eps^{-1} (s y), s = *scale_dev (1 if null)
 bec_status apply_pinv(bec_problem* p, const double* y, double* z, const double* scale_dev);
 
@@ -264,6 +286,25 @@ bec_status launch_time_pass(bec_problem* p, void* data, int fp64, double scale,
                             const double* scale_dev);
 bec_status launch_time_pass_w(bec_problem* p, void* data, int fp64, double scale,
                               const double* scale_dev, int w);
+// Fixed-point passes (bec_fx_dst.cu, bec_fx_time.cu).  fx_wanted: the sizes
+// and options they take (FP64 sine-transform route, n >= 32, N >= 32).
+bool fx_wanted(const bec_problem_desc* d, int logn, int logt);
+// allocates the tables; on failure nothing stays allocated and the problem
+// runs the floating-point passes
+bec_status fx_setup(bec_problem* p);
+bec_status fx_set_eps(bec_problem* p, const std::vector<double>& es);
+void fx_free(bec_problem* p);
+// tiles of 2 lpb points in a row of m
+inline int fx_xg(const bec_problem* p) {
+  const int xg = (p->m + 1) / (2 * p->fx.lpb);
+  return xg > 0 ? xg : 1;
+}
+inline bool fx_applies(const bec_problem* p) { return p->fx.q != nullptr; }
+// x-DST of every row (forward: FP64 in, integers out; back: integers in, FP64
+// out), column DSTs and time pass on integers, in place
+bec_status launch_fx_rows(bec_problem* p, const double* in, double* out, bool forward);
+bec_status launch_fx_cols(bec_problem* p, double* data, bool forward);
+bec_status launch_fx_time(bec_problem* p, double* data, const double* scale_dev);
 // rinv64[q][k] = 1 / |lambda'_k + tau mu_q|^2 from the current lambda' table
 bec_status launch_rinv_table(bec_problem* p);
 // y = x converted between FP64 and FP32 (to_float: double -> float) by the

@@ -94,7 +94,8 @@ bec_status autotune(bec_problem* p, int force, bec_tune_report* rep) {
   const int fp64 = p->desc.precision == BEC_PC_FP64;
   const int tsize = fp64 ? 8 : 4;
   const Key key{fp64, p->dim, p->m, p->N};
-  if (p->desc.route != BEC_ROUTE_FST) {   // the other routes have no tunable pass
+  // the other routes and the fixed-point passes have no tunable width
+  if (p->desc.route != BEC_ROUTE_FST) {
     if (rep) *rep = r;
     return BEC_OK;
   }
@@ -119,7 +120,7 @@ bec_status autotune(bec_problem* p, int force, bec_tune_report* rep) {
   BEC_CUDA_TRY(cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   double* x = p->V;
   void* s = p->pc_scratch;
-  BEC_CUDA_TRY(cudaMemsetAsync(x, 0, (size_t)p->U * sizeof(double), p->stream));
+  if (!fx_applies(p)) BEC_CUDA_TRY(cudaMemsetAsync(x, 0, (size_t)p->U * sizeof(double), p->stream));
   if (!fp64) BEC_CUDA_TRY(cudaMemsetAsync(s, 0, (size_t)p->N * p->Jp * sizeof(float), p->stream));
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   BEC_CUDA_TRY(cudaEventCreate(&e0));
@@ -133,6 +134,7 @@ bec_status autotune(bec_problem* p, int force, bec_tune_report* rep) {
   int best[3] = {0, 0, 0};
   bec_status st = BEC_OK;
   for (int which = 0; which < 3 && st == BEC_OK; ++which) {
+    if (fx_applies(p)) continue;                  // the fixed-point passes have fixed blocks
     if (which == 1 && p->dim < 2) continue;
     if (which == 2 && time16_applies(p)) continue;   // fixed block of 8 warps
     if (which == 1 && cols16_applies(p)) continue;   // likewise
