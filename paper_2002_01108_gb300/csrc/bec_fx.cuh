@@ -556,7 +556,7 @@ BEC_FX i64 d_to_fx(u64 b, int F) {
 // v 2^F rounded to nearest (ties away from zero).  fx_to_d takes |v| >= 2^32
 // with a normal result (fx_normal(F)) itself; the rest goes through ldexp.
 static __host__ __device__ __noinline__ double fx_to_d_slow(i64 v, int F) {
-  return ldexp((double)v, F);
+  return v == 0 ? 0.0 : ldexp((double)v, F);
 }
 BEC_FX bool fx_normal(int F) { return F > -1030 && F < 950; }
 BEC_FX double fx_to_d(i64 v, int F) {

@@ -195,7 +195,6 @@ bec_status gmres_run_step(GmresRun& r, bool* enqueued) {
       } else {
         BEC_TRY(launch_norm(p, r.f, S_REF));
       }
-      if (!r.o.use_x0) BEC_TRY(launch_zero(p, r.u));
       BEC_TRY(enqueue_scalar_read(p));
       r.state = GmresRun::AFTER_BEGIN;
       *enqueued = true;
@@ -204,6 +203,7 @@ bec_status gmres_run_step(GmresRun& r, bool* enqueued) {
     case GmresRun::AFTER_BEGIN: {
       r.ref = p->host_scal[S_REF];
       if (!std::isfinite(r.ref)) {
+        if (!r.x_nonzero) BEC_TRY(launch_zero(p, r.u));
         set_error("right-hand side contains NaN or Inf");
         r.state = GmresRun::DONE;
         return r.status = BEC_ENUMERIC;
@@ -242,6 +242,7 @@ bec_status gmres_run_step(GmresRun& r, bool* enqueued) {
     case GmresRun::AFTER_CYCLE: {
       const double beta = r.beta_slot == S_BETA ? p->host_scal[S_BETA] : r.ref;
       if (!std::isfinite(beta)) {
+        if (!r.x_nonzero) BEC_TRY(launch_zero(p, r.u));
         set_error("NaN or Inf in the GMRES residual");
         r.state = GmresRun::DONE;
         return r.status = BEC_ENUMERIC;
@@ -273,6 +274,7 @@ bec_status gmres_run_step(GmresRun& r, bool* enqueued) {
       ++r.iters;
       r.k = r.j + 1;
       if (!std::isfinite(res)) {
+        if (!r.x_nonzero) BEC_TRY(launch_zero(p, r.u));
         set_error("NaN or Inf in the GMRES recurrences");
         r.state = GmresRun::DONE;
         return r.status = BEC_ENUMERIC;
@@ -288,15 +290,16 @@ bec_status gmres_run_step(GmresRun& r, bool* enqueued) {
       // end of the cycle: least squares and the solution update
       BEC_TRY(launch_least_squares(p, r.k));
       double* sigma = p->sigma;
+      const double* u0 = r.x_nonzero ? r.u : nullptr;   // the first update writes u
       if (r.o.left_pc) {
-        BEC_TRY(launch_combine(p, r.u, r.u, r.Vp.data(), r.k, sigma, p->ycoef, 1.0, -1));
+        BEC_TRY(launch_combine(p, r.u, u0, r.Vp.data(), r.k, sigma, p->ycoef, 1.0, -1));
       } else if (r.o.flexible) {
-        BEC_TRY(launch_combine(p, r.u, r.u, r.Zp.data(), r.k, nullptr, p->ycoef, 1.0, -1));
+        BEC_TRY(launch_combine(p, r.u, u0, r.Zp.data(), r.k, nullptr, p->ycoef, 1.0, -1));
       } else {
         BEC_TRY(launch_combine(p, p->t, nullptr, r.Vp.data(), r.k, sigma, p->ycoef, 1.0, -1));
         BEC_TRY(apply_pinv(p, p->t, p->w, nullptr));
         const double* wl[1] = {p->w};
-        BEC_TRY(launch_combine(p, r.u, r.u, wl, 1, nullptr, p->scal + S_ONE, 1.0, -1));
+        BEC_TRY(launch_combine(p, r.u, u0, wl, 1, nullptr, p->scal + S_ONE, 1.0, -1));
       }
       r.x_nonzero = true;
       if (stop) {
@@ -308,7 +311,8 @@ bec_status gmres_run_step(GmresRun& r, bool* enqueued) {
       return BEC_OK;
     }
     case GmresRun::FINISH: {
-      BEC_TRY(launch_residual_norms(p, r.f, r.u, S_TRUE));
+      if (!r.x_nonzero) BEC_TRY(launch_zero(p, r.u));   // no update was needed
+      BEC_TRY(launch_residual_norms(p, r.f, r.u, S_TRUE, r.o.left_pc ? -1 : S_REF));
       BEC_TRY(enqueue_scalar_read(p));
       r.state = GmresRun::AFTER_FINISH;
       *enqueued = true;

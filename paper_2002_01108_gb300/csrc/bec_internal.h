@@ -465,8 +465,9 @@ bec_status launch_build_rhs(bec_problem* p, const double* u0,
                             const double* fsrc, double* f);
 // partials[b] = sum over block b of (f - L u)^2, partials[B + b] = sum f^2;
 // then scal[slot] = sqrt(sum r^2), scal[slot+1] = sqrt(sum f^2).
+// fslot >= 0: ||f|| is in scal[fslot] and is copied instead.
 bec_status launch_residual_norms(bec_problem* p, const double* f,
-                                 const double* u, int slot);
+                                 const double* u, int slot, int fslot = -1);
 // r = f - L u (u may be null: r = f)
 bec_status launch_residual(bec_problem* p, const double* f, const double* u,
                            double* r);

@@ -112,7 +112,10 @@ update_dots_kernel(double* __restrict__ w, VecList V, long long U, const double*
   block_store_dots<NV>(acc, partials);
 }
 
-// out = w + sign sum_{v<nv} coef_v sigma_v V_v (w null: 0); optional sum of out^2.
+// out = w + sign sum_{v<nv} coef_v sigma_v V_v (w null: 0); NORM: sum of out^2.
+// Bound by the FP64 pipe (nv operations an element, one more for the norm) about
+// as much as by the vectors' traffic.
+template <bool NORM>
 __global__ void __launch_bounds__(kThreads)
 combine_kernel(double* out, const double* w, VecList V, int nv, long long U,
                const double* __restrict__ coef, const double* __restrict__ sigma, double sign,
@@ -134,9 +137,9 @@ combine_kernel(double* out, const double* w, VecList V, int nv, long long U,
       a.y = fma(c[v], x.y, a.y);
     }
     o2[i] = a;
-    nrm = fma(a.x, a.x, fma(a.y, a.y, nrm));
+    if (NORM) nrm = fma(a.x, a.x, fma(a.y, a.y, nrm));
   }
-  if (partials != nullptr) block_store_sum(nrm, partials);
+  if (NORM) block_store_sum(nrm, partials);
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -349,7 +352,7 @@ bec_status launch_combine(bec_problem* p, double* out, const double* w, const do
     double* part = (last && norm_slot >= 0) ? p->partials : nullptr;
     const double* src = v0 == 0 ? w : out;
     BEC_LAUNCH_BEGIN(p);
-    combine_kernel<<<kReduceBlocks, kThreads, 0, p->stream>>>(
+    (part != nullptr ? combine_kernel<true> : combine_kernel<false>)<<<kReduceBlocks, kThreads, 0, p->stream>>>(
         out, src, pack(V + v0, n > 0 ? n : 1), n, p->U, coef + v0, sigma ? sigma + v0 : nullptr,
         sign, part, flag);
     BEC_LAUNCH_CHECK(p, "combine_kernel");

@@ -14,6 +14,9 @@
 // v^{n-1} in a register, so v is read from memory once.
 #include <cuda_runtime.h>
 
+#include <cmath>
+
+#include "bec_fx.cuh"
 #include "bec_internal.h"
 
 namespace bec {
@@ -369,8 +372,9 @@ residual_norms_kernel(const double* __restrict__ f, const double* __restrict__ u
   }
 }
 
+// fslot >= 0: ||f|| is scal[fslot] already
 __global__ void finish_norms_kernel(const double* __restrict__ partials, long long nblk,
-                                    double* __restrict__ scal, int slot) {
+                                    double* __restrict__ scal, int slot, int fslot) {
   __shared__ double s_a[256], s_b[256];
   double a = 0.0, b = 0.0;
   for (long long i = threadIdx.x; i < nblk; i += blockDim.x) {
@@ -389,7 +393,7 @@ __global__ void finish_norms_kernel(const double* __restrict__ partials, long lo
   }
   if (threadIdx.x == 0) {
     scal[slot] = sqrt(s_a[0]);
-    scal[slot + 1] = sqrt(s_b[0]);
+    scal[slot + 1] = fslot >= 0 ? scal[fslot] : sqrt(s_b[0]);
   }
 }
 
@@ -415,6 +419,273 @@ __global__ void build_rhs_kernel(const double* __restrict__ u0, const double* __
       v = coef == 1.0 ? v + mu : fma(coef, mu, v);
     }
     f[i] = v;
+  }
+}
+
+// ---------------------------------------------------------------- fixed point
+// The finite-difference rows of L in 64-bit fixed point (bec_fx.cuh), 2D and
+// 3D with a constant coefficient.
+//
+// GB300 issues 2 FP64 operations a clock and SM: the 5 (2D) or 7 (3D) of a row
+// bound the kernels above, whose vectors' traffic takes a quarter of that time.
+// Here a row is integer work: L v = c (2 dim v - sum of neighbours) + v - v^{n-1}
+// with the differences exact, one product by c and one conversion to FP64; the
+// FP64 pipe keeps only what follows (the shift, the dots, the norms).
+//
+// A warp owns 32 columns and kFxRows rows of one slice (3D: of one plane) and
+// walks a chunk of time steps.  A lane converts its rows and the two beside
+// them once and gets its x neighbours by shuffle; only the edge lanes load one
+// more value a row.  The unit is a power of two from the largest value the
+// warp has loaded for the step and the one before, so that |v| < 2^59: the
+// error is below 2^-55 c max|v| of the tile, less than an FP64 row's.  Values
+// that are not finite or leave the range go through the FP64 row.
+// Measured at 255^2 x 256: w = L z - s v with 1 and 2 dots 161 us on average
+// (FP64 rows: 287), ||f - L u|| 116 us (300); what bounds them now is the FP64
+// pipe again (2 operations and one a dot), 70 to 80 % busy.
+constexpr int kFxRows = 4;
+constexpr int kFxDotVecs = 8;        // vectors a fused launch takes; more go to dots_kernel
+
+struct FxStencil {
+  fx::W64 cm;      // c = cm 2^-63 2^ce
+  int ce;
+  int chunk;       // time steps of a tile
+  int xt, yg, planes;   // tiles in x, row groups, planes (3D: m)
+  int tiles;
+};
+
+enum { kModeDots = 0, kModeNorms = 1, kModeApply = 2, kModeResidual = 3 };
+
+// the FP64 row at point q of the slice vs = v^n
+template <int KIND, int P>
+__device__ __noinline__ double fx_slow_row(const double* __restrict__ vs, long long q, int ix, int iy, int iz,
+                                           int n, const StencilGeom& g) {
+  return row_of<KIND, P>(vs, nullptr, nullptr, q, ix, iy, iz, g, vs[q], n > 0 ? vs[q - g.J] : 0.0,
+                         P == 2 && n > 1 ? vs[q - 2 * g.J] : 0.0);
+}
+
+template <int KIND, int P>
+struct FxRow {
+  static constexpr int R = kFxRows;
+  static constexpr bool D3 = KIND == kFD3;
+  // one slice's values of the tile, as bit patterns (zeros outside the domain)
+  struct Raw {
+    fx::u64 b[R + 2];        // the lane's column: the row below, the rows, the row above
+    fx::u64 edge;            // lane r < R: left of row r; lane R + r: right of it
+    fx::u64 d[D3 ? R : 1], u[D3 ? R : 1];   // 3D: the planes below and above
+  };
+  int m, lane, x, y0, z0, rows;
+  unsigned in;               // which of b[] lie inside the domain; bit 31: the edge value
+  long long q0, eo;          // the lane's first row; its edge value's point
+  fx::i64 prev[R], prev2[P == 2 ? R : 1];
+  int Fp, Fp2, ep, ep2;      // unit and largest exponent field of prev, prev2
+
+  __device__ __forceinline__ void start(const StencilGeom& g, const FxStencil& f, int t, int ln) {
+    lane = ln;
+    m = g.m;
+    const int a = t / f.xt, x0 = (t - a * f.xt) * 32;
+    z0 = D3 ? a / f.yg : 0;
+    y0 = (a - z0 * f.yg) * R;
+    x = x0 + lane;
+    rows = min(R, m - y0);
+    q0 = ((long long)z0 * m + y0) * m + x;
+    in = 0;
+    if (x < m) {
+      in = ((1u << rows) - 1u) << 1;
+      if (y0 > 0) in |= 1u;
+      if (y0 + rows < m) in |= 1u << (rows + 1);
+    }
+    const int er = lane % R, ex = lane < R ? x0 - 1 : x0 + 32;
+    if (lane < 2 * R && er < rows && ex >= 0 && ex < m) in |= 1u << 31;
+    eo = ((long long)z0 * m + y0 + er) * m + ex;
+  }
+  __device__ __forceinline__ bool row_in(int r) const { return in >> (r + 1) & 1; }
+  __device__ __forceinline__ void load(const double* __restrict__ vs, Raw& w) const {
+    const double* p = vs + q0;
+#pragma unroll
+    for (int r = 0; r < R + 2; ++r) w.b[r] = in >> r & 1 ? fx::d_bits(p[(r - 1) * m]) : 0;
+    w.edge = in >> 31 ? fx::d_bits(vs[eo]) : 0;
+    if constexpr (D3) {
+      const long long m2 = (long long)m * m;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        w.d[r] = row_in(r) && z0 > 0 ? fx::d_bits(p[r * m - m2]) : 0;
+        w.u[r] = row_in(r) && z0 + 1 < m ? fx::d_bits(p[r * m + m2]) : 0;
+      }
+    }
+  }
+  // the centre values of a slice (zeros where there is none)
+  __device__ __forceinline__ void load_prev(const double* __restrict__ vs, fx::i64 (&pv)[R], int& F, int& e) {
+    fx::u64 b[R];
+    int h = 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      b[r] = vs != nullptr && row_in(r) ? fx::d_bits(vs[q0 + r * m]) : 0;
+      h = max(h, fx::d_habs(b[r]));
+    }
+    e = (int)__reduce_max_sync(0xffffffffu, (unsigned)h) >> 20;
+    F = max(e - 1081, fx::kFxMin);
+#pragma unroll
+    for (int r = 0; r < R; ++r) pv[r] = fx::d_to_fx(b[r], F);
+  }
+  // y = row values of the slice vs = v^n, whose values are in w
+  __device__ __forceinline__ void step(const Raw& w, const double* __restrict__ vs, const StencilGeom& g,
+                                       const FxStencil& f, int n, double (&y)[R]) {
+    using fx::i64;
+    int h = fx::d_habs(w.edge);
+#pragma unroll
+    for (int r = 0; r < R + 2; ++r) h = max(h, fx::d_habs(w.b[r]));
+    if constexpr (D3) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) h = max(h, max(fx::d_habs(w.d[r]), fx::d_habs(w.u[r])));
+    }
+    const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)h) >> 20;
+    const int em = max(max(e, ep), P == 2 ? ep2 : 0);
+    const int F = max(em - 1081, fx::kFxMin);            // |v| < 2^(em - 1022) = 2^(F + 59)
+    const int s = f.ce + 1;                               // c lap = mul64(lap, cm) 2^s
+    const int G = F + max(s, 0);
+    if (em == 0x7FF || !fx::fx_normal(G)) {
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        y[r] = row_in(r) ? fx_slow_row<KIND, P>(vs, q0 + r * m, x, y0 + r, z0, n, g) : 0.0;
+      ep = e;
+      Fp = F;
+#pragma unroll
+      for (int r = 0; r < R; ++r) prev[r] = fx::d_to_fx(w.b[r + 1], F);
+      if constexpr (P == 2) load_prev(n > 0 ? vs - g.J : nullptr, prev2, Fp2, ep2);
+      return;
+    }
+    if (F != Fp) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) prev[r] = fx::shift(prev[r], F - Fp);
+    }
+    if (P == 2 && F != Fp2) {
+#pragma unroll
+      for (int r = 0; r < (P == 2 ? R : 0); ++r) prev2[r] = fx::shift(prev2[r], F - Fp2);
+    }
+    // shifts round to nearest: a bias of even a small part of a unit, the same at
+    // every point, would come back from L^{-1} many times larger
+    const i64 rnd = s == 0 ? 0 : 1LL << (min(abs(s), 60) - 1);
+    const i64 edge = fx::d_to_fx(w.edge, F);
+    i64 below = fx::d_to_fx(w.b[0], F), c = fx::d_to_fx(w.b[1], F);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const i64 above = fx::d_to_fx(w.b[r + 2], F);
+      i64 le = __shfl_up_sync(0xffffffffu, c, 1), ri = __shfl_down_sync(0xffffffffu, c, 1);
+      const i64 ed = __shfl_sync(0xffffffffu, edge, lane < 16 ? r : R + r);
+      if (lane == 0) le = ed;
+      if (lane == 31) ri = ed;
+      i64 lap = (c << 2) - ((le + ri) + (below + above));
+      if constexpr (D3) lap += (c << 1) - (fx::d_to_fx(w.d[r], F) + fx::d_to_fx(w.u[r], F));
+      const i64 t = fx::mul64(lap, f.cm);
+      i64 Y;
+      if constexpr (P == 2) {                             // (3 v - 4 v' + v'') / 2
+        const i64 d = 3 * c - 4 * prev[r] + prev2[r];
+        Y = s >= 0 ? t + fx::shr(d + (1LL << s), s + 1) : fx::shr(t + rnd, -s) + ((d + 1) >> 1);
+        prev2[r] = prev[r];
+      } else {
+        const i64 d = c - prev[r];
+        Y = s >= 0 ? t + fx::shr(d + rnd, s) : fx::shr(t + rnd, -s) + d;
+      }
+      prev[r] = c;
+      y[r] = fx::fx_to_d(Y, G);
+      below = c;
+      c = above;
+    }
+    if constexpr (P == 2) {
+      ep2 = ep;
+      Fp2 = F;
+    }
+    ep = e;
+    Fp = F;
+  }
+};
+
+// z: the vector the rows apply to.  kModeDots: w = L z - s vshift, partials as
+// stencil_dots_kernel (LAST: vshift is V_{NV-1}); kModeNorms: partials as
+// residual_norms_kernel (aux = f; LAST: without f^2); kModeApply: w = L z (times *sshift if
+// given); kModeResidual: w = aux - L z.
+template <int MODE, int NV, bool LAST, int KIND, int P>
+__global__ void __launch_bounds__(kStencilThreads, NV <= 2 && KIND != kFD3 ? 3 : 2)
+stencil_fx_kernel(const double* __restrict__ z, const double* __restrict__ aux, double* __restrict__ w,
+                  StencilGeom g, FxStencil f, VecList V, const double* __restrict__ vshift,
+                  const double* __restrict__ sshift, double* __restrict__ partials) {
+  using Row = FxRow<KIND, P>;
+  constexpr int R = kFxRows, NA = MODE == kModeDots ? NV + 1 : 2;
+  double acc[NA];
+#pragma unroll
+  for (int v = 0; v < NA; ++v) acc[v] = 0.0;
+  const int lane = threadIdx.x & 31;
+  const double ss = sshift ? sshift[0] : (MODE == kModeApply ? 1.0 : 0.0);
+  const int wstep = gridDim.x * (kStencilThreads / 32), per = f.xt * f.yg * f.planes;
+  Row row;
+  for (int t = blockIdx.x * (kStencilThreads / 32) + (threadIdx.x >> 5); t < f.tiles; t += wstep) {
+    const int tc = t / per;
+    row.start(g, f, t - tc * per, lane);
+    const int n0 = tc * f.chunk, n1 = min(g.N, n0 + f.chunk);
+    const double* zs = z + (long long)n0 * g.J;
+    typename Row::Raw cur, nxt;
+    row.load(zs, cur);
+    row.load_prev(n0 > 0 ? zs - g.J : nullptr, row.prev, row.Fp, row.ep);
+    if constexpr (P == 2)
+      row.load_prev(n0 > 1 ? zs - 2 * g.J : nullptr, row.prev2, row.Fp2, row.ep2);
+    long long o0 = (long long)n0 * g.J + row.q0;
+    for (int n = n0; n < n1; ++n) {
+      // the next slice's values and this one's other operands are on their way
+      // while this slice is worked on
+      if (n + 1 < n1) row.load(zs + g.J, nxt);
+      double a1[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        a1[r] = 0.0;
+        if (!row.row_in(r)) continue;
+        if constexpr (MODE == kModeDots) a1[r] = LAST ? V.v[NV - 1][o0 + r * g.m] : vshift ? vshift[o0 + r * g.m] : 0.0;
+        else if constexpr (MODE != kModeApply) a1[r] = aux[o0 + r * g.m];
+      }
+      double y[R];
+      row.step(cur, zs, g, f, n, y);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        if (!row.row_in(r)) continue;
+        const long long o = o0 + r * g.m;
+        if constexpr (MODE == kModeDots) {
+          const double a = fma(-ss, a1[r], y[r]);
+          w[o] = a;
+#pragma unroll
+          for (int v = 0; v < NV; ++v) acc[v] = fma(LAST && v == NV - 1 ? a1[r] : V.v[v][o], a, acc[v]);
+          acc[NV] = fma(a, a, acc[NV]);
+        } else if constexpr (MODE == kModeNorms) {
+          const double a = a1[r] - y[r];
+          acc[0] = fma(a, a, acc[0]);
+          if (!LAST) acc[1] = fma(a1[r], a1[r], acc[1]);
+        } else if constexpr (MODE == kModeApply) {
+          w[o] = sshift ? ss * y[r] : y[r];
+        } else {
+          w[o] = a1[r] - y[r];
+        }
+      }
+      zs += g.J;
+      o0 += g.J;
+      cur = nxt;
+    }
+  }
+  if constexpr (MODE == kModeDots || MODE == kModeNorms) {
+    __shared__ double red[kStencilThreads / 32][NA];
+    const int warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int v = 0; v < NA; ++v) {
+      double s = acc[v];
+      for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+      if (lane == 0) red[warp][v] = s;
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < NA) {
+      double s = 0.0;
+#pragma unroll
+      for (int wi = 0; wi < kStencilThreads / 32; ++wi) s += red[wi][threadIdx.x];
+      // dots: row v of the partials; norms: pairs
+      partials[MODE == kModeDots ? (long long)threadIdx.x * gridDim.x + blockIdx.x
+                                 : 2LL * blockIdx.x + threadIdx.x] = s;
+    }
   }
 }
 
@@ -496,6 +767,49 @@ void stencil_dots_launch(int var, cudaStream_t st, const double* z, double* w,
 #undef BEC_SD_LAUNCH
 }
 
+// The fixed-point rows take finite differences with a constant coefficient in 2D
+// and 3D from 31 points a side (a warp's 32 columns are then nearly full).
+bool fx_rows(const bec_problem* p) {
+  return p->kcoef == nullptr && p->desc.space == BEC_SPACE_FD && p->dim >= 2 && p->m >= 31;
+}
+
+// blocks: what the card holds at once (3 a SM), or fewer
+unsigned fx_stencil(const bec_problem* p, const StencilGeom& g, FxStencil& f) {
+  int ce;
+  const double cm = std::frexp(g.c, &ce);
+  long long w = (long long)std::ldexp(cm, 63);
+  if (w > 0x7FFFFFFF00000000LL) {                 // next to 1: half of it
+    w >>= 1;
+    ++ce;
+  }
+  f.cm = fx::split64(w);
+  f.ce = ce;
+  f.xt = (p->m + 31) / 32;
+  f.yg = (p->m + kFxRows - 1) / kFxRows;
+  f.planes = p->dim == 3 ? p->m : 1;
+  const int per = f.xt * f.yg * f.planes;          // at most 2^23
+  const long long warps = 3LL * 152 * (kStencilThreads / 32);
+  // the longest chunk that still gives every warp of the card a tile
+  f.chunk = 16;
+  while (f.chunk > 1 && (long long)per * ((p->N + f.chunk - 1) / f.chunk) < warps) f.chunk /= 2;
+  f.tiles = per * ((p->N + f.chunk - 1) / f.chunk);
+  const int blocks = (f.tiles + kStencilThreads / 32 - 1) / (kStencilThreads / 32);
+  return (unsigned)(blocks < 3 * 152 ? blocks : 3 * 152);
+}
+
+template <int MODE, int NV, bool LAST = false>
+void stencil_fx_launch(const bec_problem* p, unsigned grid, const double* z, const double* aux, double* w,
+                       const StencilGeom& g, const FxStencil& f, const VecList& L, const double* vshift,
+                       const double* sshift) {
+#define BEC_SFX(K, P)                                                                       \
+  stencil_fx_kernel<MODE, NV, LAST, K, P><<<grid, kStencilThreads, 0, p->stream>>>(               \
+      z, aux, w, g, f, L, vshift, sshift, p->partials)
+  if (p->dim == 3) BEC_SFX(kFD3, 1);
+  else if (p->desc.time_scheme == BEC_TIME_BDF2) BEC_SFX(kFD, 2);
+  else BEC_SFX(kFD, 1);
+#undef BEC_SFX
+}
+
 dim3 stencil_grid(const bec_problem* p) {
   return dim3((unsigned)((p->J + kStencilThreads - 1) / kStencilThreads),
               (unsigned)((p->N + kTimeChunk - 1) / kTimeChunk));
@@ -511,6 +825,14 @@ long long stencil_blocks(const bec_problem* p) {
 bec_status launch_apply_L(bec_problem* p, const double* v, double* y, double corner,
                           const double* out_scale) {
   const StencilGeom g = geom(p);
+  if (corner == 0.0 && fx_rows(p)) {
+    FxStencil f;
+    const unsigned grid = fx_stencil(p, g, f);
+    BEC_LAUNCH_BEGIN(p);
+    stencil_fx_launch<kModeApply, 1>(p, grid, v, nullptr, y, g, f, VecList{}, nullptr, out_scale);
+    BEC_LAUNCH_CHECK(p, "apply_L_fx_kernel");
+    return BEC_OK;
+  }
   BEC_LAUNCH_BEGIN(p);
 #define BEC_L_LAUNCH(K, P)                                                \
   apply_L_kernel<K, P><<<stencil_grid(p), kStencilThreads, 0, p->stream>>>( \
@@ -525,11 +847,33 @@ bec_status launch_stencil_dots(bec_problem* p, const double* z, double* w,
                                const double* const* V, int nv, const double* sigma,
                                double* hout, const double* vshift, const double* sshift,
                                int norm_slot) {
-  const int n = nv < kMaxVec ? nv : kMaxVec;
+  const bool fixed = fx_rows(p);
+  const int most = fixed ? kFxDotVecs : kMaxVec, n = nv < most ? nv : most;
   VecList L;
   for (int i = 0; i < kMaxVec; ++i) L.v[i] = i < n ? V[i] : V[0];
   const int var = variant_of(p);
   const StencilGeom g = geom(p);
+  int nb = kStencilDotBlocks;
+  if (fixed) {
+    FxStencil f;
+    const unsigned grid = fx_stencil(p, g, f);
+    nb = (int)grid;
+    BEC_LAUNCH_BEGIN(p);
+    switch (n) {
+#define BEC_SFX_CASE(NV)                                                                    \
+  case NV:                                                                                  \
+    if (vshift == V[NV - 1])                                                                \
+      stencil_fx_launch<kModeDots, NV, true>(p, grid, z, nullptr, w, g, f, L, vshift, sshift);  \
+    else                                                                                    \
+      stencil_fx_launch<kModeDots, NV>(p, grid, z, nullptr, w, g, f, L, vshift, sshift);    \
+    break;
+      BEC_SFX_CASE(1) BEC_SFX_CASE(2) BEC_SFX_CASE(3) BEC_SFX_CASE(4) BEC_SFX_CASE(5) BEC_SFX_CASE(6)
+      BEC_SFX_CASE(7) BEC_SFX_CASE(8)
+#undef BEC_SFX_CASE
+      default: return BEC_EINVAL;
+    }
+    BEC_LAUNCH_CHECK(p, "stencil_dots_fx_kernel");
+  } else {
   BEC_LAUNCH_BEGIN(p);
   switch (n) {
 #define BEC_SD_CASE(NV)                                                                  \
@@ -546,21 +890,28 @@ bec_status launch_stencil_dots(bec_problem* p, const double* z, double* w,
     default: return BEC_EINVAL;
   }
   BEC_LAUNCH_CHECK(p, "stencil_dots_kernel");
+  }
   bec_status s = BEC_OK;
   if (norm_slot >= 0) {
-    s = launch_finish_sqrt(p, p->partials + (long long)n * kStencilDotBlocks, kStencilDotBlocks,
-                           norm_slot, nullptr);
+    s = launch_finish_sqrt(p, p->partials + (long long)n * nb, nb, norm_slot, nullptr);
     if (s != BEC_OK) return s;
   }
-  s = launch_finish_dots(p, n, kStencilDotBlocks, sigma, hout);
-  if (s != BEC_OK || nv <= kMaxVec) return s;
+  s = launch_finish_dots(p, n, nb, sigma, hout);
+  if (s != BEC_OK || nv <= most) return s;
   // more vectors than one fused launch holds: the rest as plain dots
-  return launch_dots(p, w, V + kMaxVec, nv - kMaxVec, sigma ? sigma + kMaxVec : nullptr,
-                     hout + kMaxVec);
+  return launch_dots(p, w, V + most, nv - most, sigma ? sigma + most : nullptr, hout + most);
 }
 
 bec_status launch_residual(bec_problem* p, const double* f, const double* u, double* r) {
   const StencilGeom g = geom(p);
+  if (u != nullptr && fx_rows(p)) {
+    FxStencil x;
+    const unsigned grid = fx_stencil(p, g, x);
+    BEC_LAUNCH_BEGIN(p);
+    stencil_fx_launch<kModeResidual, 1>(p, grid, u, f, r, g, x, VecList{}, nullptr, nullptr);
+    BEC_LAUNCH_CHECK(p, "residual_fx_kernel");
+    return BEC_OK;
+  }
   BEC_LAUNCH_BEGIN(p);
 #define BEC_R_LAUNCH(K, P) \
   residual_kernel<K, P><<<stencil_grid(p), kStencilThreads, 0, p->stream>>>(f, u, r, g)
@@ -570,18 +921,30 @@ bec_status launch_residual(bec_problem* p, const double* f, const double* u, dou
   return BEC_OK;
 }
 
-bec_status launch_residual_norms(bec_problem* p, const double* f, const double* u, int slot) {
+bec_status launch_residual_norms(bec_problem* p, const double* f, const double* u, int slot, int fslot) {
   const dim3 grid = stencil_grid(p);
   const StencilGeom g = geom(p);
+  long long nblk = (long long)grid.x * grid.y;
+  if (fx_rows(p)) {
+    FxStencil x;
+    const unsigned gx = fx_stencil(p, g, x);
+    nblk = gx;
+    BEC_LAUNCH_BEGIN(p);
+    if (fslot >= 0)
+      stencil_fx_launch<kModeNorms, 1, true>(p, gx, u, f, nullptr, g, x, VecList{}, nullptr, nullptr);
+    else
+      stencil_fx_launch<kModeNorms, 1>(p, gx, u, f, nullptr, g, x, VecList{}, nullptr, nullptr);
+    BEC_LAUNCH_CHECK(p, "residual_norms_fx_kernel");
+  } else {
   BEC_LAUNCH_BEGIN(p);
 #define BEC_RN_LAUNCH(K, P) \
   residual_norms_kernel<K, P><<<grid, kStencilThreads, 0, p->stream>>>(f, u, p->partials, g)
   BEC_STENCIL_SWITCH(variant_of(p), BEC_RN_LAUNCH)
 #undef BEC_RN_LAUNCH
   BEC_LAUNCH_CHECK(p, "residual_norms_kernel");
+  }
   BEC_LAUNCH_BEGIN(p);
-  finish_norms_kernel<<<1, 256, 0, p->stream>>>(p->partials, (long long)grid.x * grid.y, p->scal,
-                                                 slot);
+  finish_norms_kernel<<<1, 256, 0, p->stream>>>(p->partials, nblk, p->scal, slot, fslot);
   BEC_LAUNCH_CHECK(p, "finish_norms_kernel");
   return BEC_OK;
 }
