@@ -4,7 +4,7 @@
 // The division by lambda'_k + tau mu is a product by a table of reciprocals in
 // fixed point (16 bytes a mode and frequency, 8 bytes an unknown read from
 // HBM); computing them would take FP64 operations.  Measured at 255^2 x 256:
-// 190 us, where the floating-point pass takes 1042 us.
+// 189 us, where the floating-point pass takes 1042 us.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -168,9 +168,13 @@ bool fx_wanted(const bec_problem_desc* d, int logn, int logt) {
 bec_status fx_setup(bec_problem* p) {
   FxTables& t = p->fx;
   const int n = p->m + 1, N = p->N;
-  // 16 line pairs a block; 8 for the long lines whose blocks would otherwise
-  // pass 512 threads
-  t.lpb = p->tab.space.logn >= 9 || p->tab.time.logn >= 9 ? 8 : 16;
+  // 16 line pairs a block (256-byte segments across the lines); 8 for the long
+  // lines whose blocks would otherwise pass 512 threads, and where both passes
+  // still have 64 threads a block with 8: more and smaller blocks overlap
+  // better there (255^2 x 256: 581 against 614 us an apply), while shorter
+  // lines lose (63^3 x 64: 733 against 671 us)
+  t.lpb = p->tab.space.logn >= 9 || p->tab.time.logn >= 9 || (p->tab.space.logn == 8 && p->tab.time.logn >= 7)
+              ? 8 : 16;
   // one exponent a tile: of rows, and of columns or modes
   const long long units = p->J / p->m, tiles = units * fx_xg(p);
   const long long ne = std::max((units * N + 2 * t.lpb - 1) / (2 * t.lpb),
