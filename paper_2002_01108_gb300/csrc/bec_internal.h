@@ -98,8 +98,8 @@ struct MgLevel {
   void* x = nullptr;    // [K][J] complex
   void* b = nullptr;
   void* r = nullptr;
-  void* dinv = nullptr; // [K][J] complex: 1 / D of the ILU smoother (BEC_MG_ILU)
-  void* ilu_nb = nullptr;   // [2][J][8] real: the M and K entries towards the lower
+  void* dinv = nullptr; // [K][J] complex (FP32: wavefront order): 1 / D of the ILU smoother (BEC_MG_ILU)
+  void* ilu_nb = nullptr;   // [2][J][8] real, in the order of dinv: the M and K entries towards the lower
                             // (W, S, SE, SW) and upper (E, N, NW, NE) neighbours
 };
 
@@ -109,6 +109,8 @@ struct MgState {
   int ilu = 0;          // smoother: 0 damped Jacobi, 1 ILU
   int K = 0;            // N/2 + 1 frequencies
   std::vector<MgLevel> lv;
+  void* yw = nullptr;   // [K][J of the finest level] complex, or null: the ILU row kernel's
+                        // intermediate, in wavefront order (levels take turns)
 };
 
 struct NetState;   // learned correction (bec_net.cu)
@@ -327,6 +329,9 @@ bec_status mg_ilu_setup(bec_problem* p);
 // f = tau (fsrc - K_b g) + u0 in slice 1 (multigrid route)
 bec_status launch_build_rhs_dirichlet(bec_problem* p, const double* u0, const double* fsrc,
                                       const double* g, double* f);
+// the buffer of the ILU row kernel, as large as the finest level; without the
+// memory for it the wavefront kernel works in place
+void mg_alloc_spare(bec_problem* p);
 void mg_free(bec_problem* p);
 // One V-cycle for every frequency: level-0 b -> level-0 x.
 bec_status mg_vcycle(bec_problem* p);

@@ -459,6 +459,18 @@ int coarse_cycle_level(const bec_problem* p, size_t vsize) {
 // stay in a shared-memory ring indexed by [t mod 4][y].
 constexpr int kIluThreads = 128;
 
+// In FP32 1/d and the neighbour entries are stored in wavefront order, so that
+// the points a warp works on at one time are adjacent in memory: point (x, y) of
+// wavefront t = x + 2 y is at wf_base(t) + y.  (The points of the wavefronts
+// before t, less the first row ylo of t.)  In FP64, where the order gains
+// nothing, they keep the grid's order and the sweep its cheaper index.
+__host__ __device__ __forceinline__ int wf_base(int t, int m) {
+  const int a = t <= 2 * m ? (t - 1) * (t - 1) / 4 : m * (m - 1) + (t - 2 * m) * (m - 1);
+  const int s = t - (m - 1);
+  const int ylo = s > 0 ? (s + 1) / 2 : 0;
+  return a + t - (s > 1 ? s * s / 4 : 0) - ylo;
+}
+
 // entry s (stencil slot (dy+1)*3 + dx+1) of row q of lambda M + tau K
 template <typename T>
 __device__ __forceinline__ v2_t<T> ilu_coef(const MgArgs<T>& a, int s, long long q, v2_t<T> lam) {
@@ -516,7 +528,7 @@ ilu_setup_kernel(v2_t<T>* __restrict__ dinv, MgArgs<T> a) {
       }
       const V di = cinv<T>(d);
       ring[(t & 3) * m + y] = di;
-      dk[q] = di;
+      dk[sizeof(T) == 4 ? wf_base(t, m) + y : q] = di;
     }
     __syncthreads();
   }
@@ -567,12 +579,12 @@ __device__ __forceinline__ void ilu_issue(unsigned char* slot, int t, const MgAr
   const int yhi = min(m - 1, t / 2);
   const int y = ylo + (int)threadIdx.x;
   if (t >= 0 && t <= 3 * (m - 1) && y <= yhi) {
-    const long long q = (long long)y * m + (t - 2 * y);
-    const unsigned char* e = reinterpret_cast<const unsigned char*>(nb + ((FWD ? 0 : a.J) + q) * 8);
+    const long long q = (long long)y * m + (t - 2 * y), wq = sizeof(T) == 4 ? wf_base(t, m) + y : q;
+    const unsigned char* e = reinterpret_cast<const unsigned char*>(nb + ((FWD ? 0 : a.J) + wq) * 8);
 #pragma unroll
     for (int i = 0; i < 8 * (int)sizeof(T) / 16; ++i) cp_async(slot + S::kNb + 16 * i, e + 16 * i, 16);
     cp_async(slot + S::kV, src + q, 2 * (int)sizeof(T));
-    cp_async(slot + S::kD, dk + q, 2 * (int)sizeof(T));
+    cp_async(slot + S::kD, dk + wq, 2 * (int)sizeof(T));
     if (!FWD && ACC) cp_async(slot + S::kX, xk + q, 2 * (int)sizeof(T));
   }
   cp_async_commit();
@@ -715,6 +727,174 @@ ilu_sweep_async_kernel(v2_t<T>* __restrict__ x, v2_t<T>* work, const v2_t<T>* ri
   cp_async_wait<0>();
 }
 
+// The same step with a row per lane, in FP32, for grids whose operand slots fit.
+//
+// The wavefront kernel above is bound by the serial chain of its 2 (3 (m - 1)
+// + 1) steps: a block barrier, index arithmetic and shared-memory reads in
+// each, about 0.36 us.  Here lane l of warp w owns row y = 32 w + l throughout
+// and is at x = t - 2 l at its warp's step t, so its west neighbour is its own
+// last value, the row below arrives by one shuffle a step (south-east now,
+// south the step before, south-west the one before that), and nothing in a
+// step branches: values off the grid are zeros.  Warp w + 1 needs the last row
+// of warp w 63 steps behind it; it runs further back by as much as makes one
+// block barrier every D steps enough, and reads that row from a ring in shared
+// memory.  The operands are staged by cp.async D - 1 steps ahead, in slots of
+// the lane's own; a step reads the next one's and forms its coefficients while
+// the recurrence of this one is in flight.  The arithmetic is the wavefront
+// kernel's, operation by operation.  The backward sweep is the forward one on
+// the mirrored grid.
+//
+// The forward result goes to a buffer of its own in wavefront order: 32 lanes
+// write and read it as one segment.  No array is read and written by the same
+// sweep: copies issued ahead into lines that the sweep also stores to waited
+// for those stores (505 us a step instead of 173), so a step that adds to x
+// leaves z in r and mg_add_kernel adds it (7 us).
+//
+// Measured, one step for 65 frequencies: 127^2 173 us (wavefront kernel 272),
+// 63^2 85 (137), 31^2 40 (70), 15^2 23 (35); 255^2, 33 frequencies 381 (635),
+// 257 frequencies 764 (1142); 511^2, 33 frequencies 1166 (2134).  About 110
+// instructions in a chain of 210 ns a step bound it.  In FP64 the two FP64
+// lanes a clock bound both kernels and the wavefront kernel keeps its place
+// (127^2: 1128 us, this one 1200).
+constexpr int kIluRing = 128;     // columns of a warp's last row kept for the next warp
+
+// asynchronous copy of BYTES (8 or 16) where `on`
+template <int BYTES>
+__device__ __forceinline__ void cp_async_if(unsigned smem, const void* gmem, bool on) {
+  if constexpr (BYTES == 16)
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p cp.async.cg.shared.global [%0], [%1], 16; }"
+                 ::"r"(smem), "l"(gmem), "r"((unsigned)on) : "memory");
+  else
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p cp.async.ca.shared.global [%0], [%1], 8; }"
+                 ::"r"(smem), "l"(gmem), "r"((unsigned)on) : "memory");
+}
+
+template <typename T, bool FWD, int D>
+__device__ __forceinline__ void ilu_rows_sweep(v2_t<T>* __restrict__ dst, const v2_t<T>* __restrict__ src,
+                                               const v2_t<T>* __restrict__ dk, const T* __restrict__ nb,
+                                               const MgArgs<T>& a, v2_t<T> lam, v2_t<T>* ring,
+                                               const int* wbase, unsigned char* slots) {
+  using V = v2_t<T>;
+  using S = IluSlot<T>;
+  const int m = a.m, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int yy = warp * 32 + lane, y = FWD ? yy : m - 1 - yy;
+  const int rows = min(32, m - warp * 32);        // of this warp
+  const int last = yy < m ? m : 0;                // x < last: a point of the lane's row
+  const long long q0 = yy < m ? (long long)y * m + (FWD ? 0 : m - 1) : 0;
+  const T* nbd = nb + (FWD ? 0 : a.J * 8);
+  const unsigned slot0 = (unsigned)__cvta_generic_to_shared(slots), step = blockDim.x * S::kBytes;
+  auto coefv = [&](T sm, T sk) -> V { return {lam.x * sm + a.tau * sk, lam.y * sm}; };
+  // starts the copies of the lane's operands at step t
+  auto issue = [&](int t, int stage) {
+    const int x = t - 2 * lane;
+    const bool on = x >= 0 && x < last;
+    const int tw = min(t + 64 * warp, 3 * (m - 1));
+    const int w = on ? wbase[FWD ? tw : 3 * (m - 1) - tw] + y : 0;
+    const unsigned sl = slot0 + stage * step;
+#pragma unroll
+    for (int i = 0; i < 8 * (int)sizeof(T) / 16; ++i)
+      cp_async_if<16>(sl + S::kNb + 16 * i, nbd + (long long)w * 8 + i * (16 / (int)sizeof(T)), on);
+    cp_async_if<2 * (int)sizeof(T)>(sl + S::kV, src + (FWD ? q0 + x : (long long)w), on);
+    cp_async_if<2 * (int)sizeof(T)>(sl + S::kD, dk + w, on);
+    cp_async_commit();
+  };
+  // one step's operands: the coefficients towards W, S, SE, SW, then value and 1/d
+  struct Op {
+    V c[4], v, d;
+  };
+  auto fetch = [&](int stage, Op& o) {
+    const unsigned char* sl = slots + (size_t)stage * step;
+    T e[8];
+    ilu_read<T>(sl, e, o.v, o.d);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) o.c[i] = coefv(e[i], e[i + 4]);
+  };
+  constexpr int LAG = (64 + D) / D;               // epochs a warp runs behind the one before
+  const int mine = (m + 2 * (nw > 1 ? 31 : m - 1) + D - 1) / D, epochs = mine + (nw - 1) * LAG;
+  V cur = {0, 0}, s1 = {0, 0}, s2 = {0, 0};       // last value; south, south-west of the next point
+  Op op;
+  for (int e = 0; e < epochs; ++e) {
+    const int le = e - warp * LAG;
+    if (le >= 0 && le < mine && rows > 0) {
+      if (le == 0) {
+        for (int i = 0; i < D - 1; ++i) issue(i, i);
+        cp_async_wait<D - 2>();
+        fetch(0, op);
+        if (warp > 0 && lane == 0) s1 = ring[(warp - 1) * kIluRing];
+      }
+#pragma unroll
+      for (int i = 0; i < D; ++i) {
+        const int t = le * D + i, x = t - 2 * lane;
+        V se;                                     // (x + 1, y - 1)
+        se.x = __shfl_up_sync(0xffffffffu, cur.x, 1);
+        se.y = __shfl_up_sync(0xffffffffu, cur.y, 1);
+        if (warp > 0) {                           // the row below lane 0's is the warp before's
+          const V rv = ring[(warp - 1) * kIluRing + ((t + 1) & (kIluRing - 1))];
+          if (lane == 0) se = t + 1 < m ? rv : V{0, 0};
+        } else if (lane == 0) {
+          se = V{0, 0};
+        }
+        issue(t + D - 1, (i + D - 1) % D);
+        cp_async_wait<D - 2>();
+        Op next;
+        fetch((i + 1) % D, next);
+        V acc = FWD ? op.v : V{0, 0};
+        const V nbv[4] = {cur, s1, se, s2};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const V c = cmul(op.c[j], nbv[j]);
+          acc.x = FWD ? acc.x - c.x : acc.x + c.x;
+          acc.y = FWD ? acc.y - c.y : acc.y + c.y;
+        }
+        const V c = cmul(acc, op.d);
+        const bool on = x >= 0 && x < last;
+        const V val = FWD ? c : V{op.v.x - c.x, op.v.y - c.y};
+        cur = on ? val : V{0, 0};
+        if (on) {
+          if (FWD) dst[wbase[t + 64 * warp] + y] = cur;
+          else dst[q0 - x] = cur;
+          if (lane == 31) ring[warp * kIluRing + (x & (kIluRing - 1))] = cur;
+        }
+        s2 = s1;
+        s1 = se;
+        op = next;
+      }
+    }
+    __syncthreads();
+  }
+  cp_async_wait<0>();
+}
+
+template <int D>
+__global__ void __launch_bounds__(D == 8 ? 256 : 512)
+ilu_rows_kernel(float2* z, float2* yw, const float2* r, const float2* __restrict__ dinv,
+                const float* __restrict__ nb, MgArgs<float> a) {
+  using T = float;
+  using V = v2_t<T>;
+  extern __shared__ __align__(16) unsigned char ilu_smem[];
+  V* ring = reinterpret_cast<V*>(ilu_smem);                       // [warps][kIluRing]
+  int* wbase = reinterpret_cast<int*>(ring + (blockDim.x >> 5) * kIluRing);
+  const int nt = 3 * (a.m - 1) + 1;
+  unsigned char* slots = reinterpret_cast<unsigned char*>(wbase + ((nt + 3) & ~3)) +
+                         (size_t)threadIdx.x * IluSlot<T>::kBytes;
+  for (int t = threadIdx.x; t < nt; t += blockDim.x) wbase[t] = wf_base(t, a.m);
+  __syncthreads();
+  const long long base = (long long)blockIdx.x * a.J;
+  const V lam = a.lam[blockIdx.x];
+  ilu_rows_sweep<T, true, D>(yw + base, r + base, dinv + base, nb, a, lam, ring, wbase, slots);
+  __syncthreads();
+  ilu_rows_sweep<T, false, D>(z + base, yw + base, dinv + base, nb, a, lam, ring, wbase, slots);
+}
+
+// x += z
+__global__ void __launch_bounds__(256) mg_add_kernel(float2* __restrict__ x, const float2* __restrict__ z,
+                                                     long long n) {
+  const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+  if (i >= n) return;
+  const float2 u = x[i], v = z[i];
+  x[i] = {u.x + v.x, u.y + v.y};
+}
+
 // ---------------------------------------------------------------- host side
 // Coarse 9-point stencil Ac = R Af P with R = P^T / 4 (layout [s][J], s =
 // (dy+1)*3 + (dx+1)).  Fine point f of a 1D grid of mf points belongs to
@@ -792,6 +972,7 @@ const char* const kResidNames[] = BEC_LV_NAMES("mg_residual_kernel");
 const char* const kRestrictNames[] = BEC_LV_NAMES("mg_restrict_kernel");
 const char* const kProlongNames[] = BEC_LV_NAMES("mg_prolong_add_kernel");
 const char* const kIluSweepNames[] = BEC_LV_NAMES("ilu_sweep_kernel");
+const char* const kIluAddNames[] = BEC_LV_NAMES("mg_add_kernel");
 const char* const kIluSetupNames[] = BEC_LV_NAMES("ilu_setup_kernel");
 #undef BEC_LV_NAMES
 
@@ -817,6 +998,34 @@ size_t ilu_sweep_smem_bytes(int m, int threads, size_t vsize) {
   return ((4 * (size_t)m * vsize + 127) & ~(size_t)127) + 4 * (size_t)threads * slot;
 }
 
+// the row kernel (FP32): a lane a row; its steps ahead (8 or 4, or 0: the slots
+// do not fit a block, and the wavefront kernel runs)
+int ilu_rows_threads(int m) { return (m + 31) / 32 * 32; }
+size_t ilu_rows_smem(int m, int depth) {
+  const size_t threads = ilu_rows_threads(m);
+  return threads / 32 * kIluRing * sizeof(float2) + (size_t)((3 * m + 4) & ~3) * 4 +
+         depth * threads * IluSlot<float>::kBytes;
+}
+int ilu_rows_depth(int m) {
+  if (m > 511) return 0;
+  for (int d : {8, 4})
+    if (ilu_rows_smem(m, d) <= 200 * 1024 && ilu_rows_threads(m) <= (d == 8 ? 256 : 512)) return d;
+  return 0;
+}
+
+template <int D>
+bec_status ilu_rows_launch(bec_problem* p, MgLevel& c, void* z, const void* rin, const MgArgs<float>& a) {
+  using V = v2_t<float>;
+  const size_t smem = ilu_rows_smem(c.m, D);
+  if (smem > 48 * 1024)
+    BEC_CUDA_TRY(cudaFuncSetAttribute(ilu_rows_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      200 * 1024));
+  ilu_rows_kernel<D><<<p->mg.K, ilu_rows_threads(c.m), smem, p->stream>>>(
+      static_cast<V*>(z), static_cast<V*>(p->mg.yw), static_cast<const V*>(rin),
+      static_cast<const V*>(c.dinv), static_cast<const float*>(c.ilu_nb), a);
+  return BEC_OK;
+}
+
 // one ILU smoothing step on level l: x = M^{-1} rin (acc false) or x += M^{-1} rin;
 // r is the work array (rin may be r)
 template <typename T>
@@ -825,6 +1034,23 @@ bec_status ilu_sweep(bec_problem* p, MgLevel& c, int l, const void* rin, bool ac
   const MgArgs<T> a = level_args<T>(p, c);
   const int threads = ilu_threads(c.m);
   const size_t smem = ilu_sweep_smem_bytes(c.m, threads, sizeof(V));
+  if constexpr (sizeof(T) == 4) {
+    const int depth = p->mg.yw ? ilu_rows_depth(c.m) : 0;
+    if (depth > 0) {
+      // x += through r, which the backward sweep no longer reads
+      void* z = acc ? c.r : c.x;
+      BEC_LAUNCH_BEGIN(p);
+      BEC_TRY_MG(depth == 8 ? ilu_rows_launch<8>(p, c, z, rin, a) : ilu_rows_launch<4>(p, c, z, rin, a));
+      BEC_LAUNCH_CHECK(p, kIluSweepNames[l]);
+      if (!acc) return BEC_OK;
+      BEC_LAUNCH_BEGIN(p);
+      const long long tot = (long long)p->mg.K * c.J;
+      mg_add_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, p->stream>>>(static_cast<V*>(c.x),
+                                                                          static_cast<const V*>(c.r), tot);
+      BEC_LAUNCH_CHECK(p, kIluAddNames[l]);
+      return BEC_OK;
+    }
+  }
   BEC_LAUNCH_BEGIN(p);
   if (acc)
     ilu_sweep_async_kernel<T, true><<<p->mg.K, threads, smem, p->stream>>>(
@@ -1097,17 +1323,20 @@ bec_status mg_setup(bec_problem* p, const double* a_nodes, const double* wind) {
     bec_status s = fp64 ? upload_stencil<double>(&L.SM, SM) : upload_stencil<float>(&L.SM, SM);
     if (s == BEC_OK) s = fp64 ? upload_stencil<double>(&L.SK, SK) : upload_stencil<float>(&L.SK, SK);
     if (s == BEC_OK && p->mg.ilu && ml > 1) {
-      // the ILU sweeps' neighbour entries, [dir][q][M W, S, SE, SW | K same]
+      // the ILU sweeps' neighbour entries, [dir][grid (FP64) or wavefront order][M W, S, SE, SW | K same]
       // (dir 0) and [M E, N, NW, NE | K same] (dir 1)
       const int lo[4] = {3, 1, 2, 0}, up[4] = {5, 7, 6, 8};
       std::vector<double> nbv((size_t)16 * L.J);
-      for (long long q = 0; q < L.J; ++q)
+      for (long long q = 0; q < L.J; ++q) {
+        const int y = (int)(q / ml), x = (int)(q - (long long)y * ml);
+        const size_t w = fp64 ? (size_t)q : (size_t)(wf_base(x + 2 * y, ml) + y);
         for (int i = 0; i < 4; ++i) {
-          nbv[(size_t)q * 8 + i] = SM[(size_t)lo[i] * L.J + q];
-          nbv[(size_t)q * 8 + 4 + i] = SK[(size_t)lo[i] * L.J + q];
-          nbv[(size_t)(L.J + q) * 8 + i] = SM[(size_t)up[i] * L.J + q];
-          nbv[(size_t)(L.J + q) * 8 + 4 + i] = SK[(size_t)up[i] * L.J + q];
+          nbv[w * 8 + i] = SM[(size_t)lo[i] * L.J + q];
+          nbv[w * 8 + 4 + i] = SK[(size_t)lo[i] * L.J + q];
+          nbv[(L.J + w) * 8 + i] = SM[(size_t)up[i] * L.J + q];
+          nbv[(L.J + w) * 8 + 4 + i] = SK[(size_t)up[i] * L.J + q];
         }
+      }
       s = fp64 ? upload_stencil<double>(&L.ilu_nb, nbv) : upload_stencil<float>(&L.ilu_nb, nbv);
     }
     const size_t bytes = (size_t)p->mg.K * L.J * csz;
@@ -1138,6 +1367,14 @@ bec_status mg_setup(bec_problem* p, const double* a_nodes, const double* wind) {
   return BEC_OK;
 }
 
+void mg_alloc_spare(bec_problem* p) {
+  if (!p->mg.ilu || p->mg.lv.empty() || p->desc.precision == BEC_PC_FP64) return;
+  if (cudaMalloc(&p->mg.yw, (size_t)p->mg.K * p->mg.lv[0].J * sizeof(float2)) != cudaSuccess) {
+    cudaGetLastError();
+    p->mg.yw = nullptr;
+  }
+}
+
 void mg_free(bec_problem* p) {
   for (MgLevel& L : p->mg.lv) {
     void* ptrs[] = {L.SM, L.SK, L.x, L.b, L.r, L.dinv, L.ilu_nb};
@@ -1145,6 +1382,8 @@ void mg_free(bec_problem* p) {
       if (q) cudaFree(q);
   }
   p->mg.lv.clear();
+  if (p->mg.yw) cudaFree(p->mg.yw);
+  p->mg.yw = nullptr;
   if (p->kcoef) cudaFree(p->kcoef);
   p->kcoef = nullptr;
   if (p->bcoef) cudaFree(p->bcoef);
