@@ -128,13 +128,6 @@ void twiddles(int n, std::vector<double2>& t64, std::vector<float2>& t32) {
   }
 }
 
-bec_status read_scalars(bec_problem* p) {
-  const bec_status s = launch_publish_scalars(p);
-  if (s != BEC_OK) return s;
-  BEC_CUDA_TRY(cudaStreamSynchronize(p->stream));
-  return BEC_OK;
-}
-
 #define BEC_TRY(expr)                  \
   do {                                 \
     bec_status _s = (expr);            \
@@ -591,8 +584,8 @@ bec_status bec_true_relres(bec_problem* p, const double* f, const double* u, dou
   if (p == nullptr || out == nullptr) return einval("null argument");
   BEC_TRY(check_vec(f));
   BEC_TRY(check_vec(u));
-  BEC_TRY(launch_residual_norms(p, f, u, S_TRUE));
-  BEC_TRY(read_scalars(p));
+  BEC_TRY(launch_residual_norms(p, f, u, S_TRUE, -1, true));
+  BEC_CUDA_TRY(cudaStreamSynchronize(p->stream));
   *out = p->host_scal[S_TRUE] / p->host_scal[S_TRUE + 1];
   return BEC_OK;
 }

@@ -25,10 +25,6 @@ constexpr int S_REF = 0, S_BETA = 1, S_W = 2, S_RES = 3, S_TRUE = 4, S_WB = 6, S
     if (_s != BEC_OK) return _s; \
   } while (0)
 
-bec_status enqueue_scalar_read(bec_problem* p) {
-  BEC_TRY(launch_publish_scalars(p));
-  return BEC_OK;
-}
 }  // namespace
 
 // z = P_eps^{-1} (s y), s = *scale_dev (1 if null)
@@ -113,9 +109,8 @@ bec_status iteration_body(GmresRun& r) {
     BEC_TRY(launch_dots(p, p->w, r.Vp.data(), j + 1, sigma, h1));
     // classical Gram-Schmidt, second pass fused with the first update
     BEC_TRY(launch_update_dots(p, p->w, r.Vp.data(), j + 1, sigma, h1, h2));
-    BEC_TRY(launch_combine(p, vnext, p->w, r.Vp.data(), j + 1, sigma, h2, -1.0, S_W));
-    BEC_TRY(launch_hessenberg(p, j, h1, h2, S_W, S_RES));
-    return enqueue_scalar_read(p);
+    BEC_TRY(launch_combine(p, vnext, p->w, r.Vp.data(), j + 1, sigma, h2, -1.0, kNormLater));
+    return launch_arnoldi_end(p, j, h1, h2, S_W, S_RES, 0.0, nullptr);
   }
   // Right preconditioning: Arnoldi on A - I with A = L P^{-1} (same Krylov
   // space, H(A) = H(A - I) + I).  w = L z_j - v_j no longer carries the
@@ -126,12 +121,10 @@ bec_status iteration_body(GmresRun& r) {
   double* z = r.o.flexible ? p->Z + (long long)j * p->U : p->t;
   if (!r.ext_pinv) BEC_TRY(apply_pinv(p, r.Vp[j], z, sigma + j));
   BEC_TRY(launch_stencil_dots(p, z, p->w, r.Vp.data(), j + 1, sigma, h1, r.Vp[j], sigma + j, S_WB));
-  BEC_TRY(launch_combine(p, vnext, p->w, r.Vp.data(), j + 1, sigma, h1, -1.0, S_W));
-  BEC_TRY(launch_reorth_flag(p, S_WB, S_W));
+  BEC_TRY(launch_combine(p, vnext, p->w, r.Vp.data(), j + 1, sigma, h1, -1.0, S_W, nullptr, S_WB));
   BEC_TRY(launch_dots(p, vnext, r.Vp.data(), j + 1, sigma, h2, p->flag));
-  BEC_TRY(launch_combine(p, vnext, vnext, r.Vp.data(), j + 1, sigma, h2, -1.0, S_W, p->flag));
-  BEC_TRY(launch_hessenberg(p, j, h1, h2, S_W, S_RES, 1.0));
-  return enqueue_scalar_read(p);
+  BEC_TRY(launch_combine(p, vnext, vnext, r.Vp.data(), j + 1, sigma, h2, -1.0, kNormLater, p->flag));
+  return launch_arnoldi_end(p, j, h1, h2, S_W, S_RES, 1.0, p->flag);
 }
 
 // Enqueue iteration j, from the problem's graph cache when graphs are used.
@@ -191,11 +184,10 @@ bec_status gmres_run_step(GmresRun& r, bool* enqueued) {
     case GmresRun::BEGIN: {   // reference norm: ||f|| (right) or ||P^{-1} f|| (left)
       if (r.o.left_pc) {
         BEC_TRY(apply_pinv(p, r.f, p->t, nullptr));
-        BEC_TRY(launch_norm(p, p->t, S_REF));
+        BEC_TRY(launch_norm(p, p->t, S_REF, true));
       } else {
-        BEC_TRY(launch_norm(p, r.f, S_REF));
+        BEC_TRY(launch_norm(p, r.f, S_REF, true));
       }
-      BEC_TRY(enqueue_scalar_read(p));
       r.state = GmresRun::AFTER_BEGIN;
       *enqueued = true;
       return BEC_OK;
@@ -232,8 +224,7 @@ bec_status gmres_run_step(GmresRun& r, bool* enqueued) {
       }
       if (r.o.left_pc) BEC_TRY(apply_pinv(p, r.x_nonzero ? p->V : r.f, p->V, nullptr));
       if (r.beta_slot == S_BETA) {
-        BEC_TRY(launch_norm(p, r.Vp[0], S_BETA));
-        BEC_TRY(enqueue_scalar_read(p));
+        BEC_TRY(launch_norm(p, r.Vp[0], S_BETA, true));
         *enqueued = true;
       }
       r.state = GmresRun::AFTER_CYCLE;
@@ -292,14 +283,14 @@ bec_status gmres_run_step(GmresRun& r, bool* enqueued) {
       double* sigma = p->sigma;
       const double* u0 = r.x_nonzero ? r.u : nullptr;   // the first update writes u
       if (r.o.left_pc) {
-        BEC_TRY(launch_combine(p, r.u, u0, r.Vp.data(), r.k, sigma, p->ycoef, 1.0, -1));
+        BEC_TRY(launch_combine(p, r.u, u0, r.Vp.data(), r.k, sigma, p->ycoef, 1.0, kNoNorm));
       } else if (r.o.flexible) {
-        BEC_TRY(launch_combine(p, r.u, u0, r.Zp.data(), r.k, nullptr, p->ycoef, 1.0, -1));
+        BEC_TRY(launch_combine(p, r.u, u0, r.Zp.data(), r.k, nullptr, p->ycoef, 1.0, kNoNorm));
       } else {
-        BEC_TRY(launch_combine(p, p->t, nullptr, r.Vp.data(), r.k, sigma, p->ycoef, 1.0, -1));
+        BEC_TRY(launch_combine(p, p->t, nullptr, r.Vp.data(), r.k, sigma, p->ycoef, 1.0, kNoNorm));
         BEC_TRY(apply_pinv(p, p->t, p->w, nullptr));
         const double* wl[1] = {p->w};
-        BEC_TRY(launch_combine(p, r.u, u0, wl, 1, nullptr, p->scal + S_ONE, 1.0, -1));
+        BEC_TRY(launch_combine(p, r.u, u0, wl, 1, nullptr, p->scal + S_ONE, 1.0, kNoNorm));
       }
       r.x_nonzero = true;
       if (stop) {
@@ -312,8 +303,7 @@ bec_status gmres_run_step(GmresRun& r, bool* enqueued) {
     }
     case GmresRun::FINISH: {
       if (!r.x_nonzero) BEC_TRY(launch_zero(p, r.u));   // no update was needed
-      BEC_TRY(launch_residual_norms(p, r.f, r.u, S_TRUE, r.o.left_pc ? -1 : S_REF));
-      BEC_TRY(enqueue_scalar_read(p));
+      BEC_TRY(launch_residual_norms(p, r.f, r.u, S_TRUE, r.o.left_pc ? -1 : S_REF, true));
       r.state = GmresRun::AFTER_FINISH;
       *enqueued = true;
       return BEC_OK;

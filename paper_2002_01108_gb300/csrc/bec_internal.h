@@ -470,9 +470,10 @@ bec_status launch_build_rhs(bec_problem* p, const double* u0,
                             const double* fsrc, double* f);
 // partials[b] = sum over block b of (f - L u)^2, partials[B + b] = sum f^2;
 // then scal[slot] = sqrt(sum r^2), scal[slot+1] = sqrt(sum f^2).
-// fslot >= 0: ||f|| is in scal[fslot] and is copied instead.
+// fslot >= 0: ||f|| is in scal[fslot] and is copied instead; to_host: as launch_norm.
 bec_status launch_residual_norms(bec_problem* p, const double* f,
-                                 const double* u, int slot, int fslot = -1);
+                                 const double* u, int slot, int fslot = -1,
+                                 bool to_host = false);
 // r = f - L u (u may be null: r = f)
 bec_status launch_residual(bec_problem* p, const double* f, const double* u,
                            double* r);
@@ -484,44 +485,41 @@ bec_status launch_residual(bec_problem* p, const double* f, const double* u,
 bec_status launch_dots(bec_problem* p, const double* w, const double* const* V,
                        int nv, const double* sigma, double* hout,
                        const int* flag = nullptr);
-// scal[slot] = sqrt(sum of nb partials) (skipped when flag && !*flag)
-bec_status launch_finish_sqrt(bec_problem* p, const double* parts, int nb, int slot,
-                              const int* flag);
-// *flag = (scal[after] < scal[before] / sqrt(2)): the second Gram-Schmidt pass
-// is needed (the test of Daniel, Gragg, Kaufman and Stewart)
-bec_status launch_reorth_flag(bec_problem* p, int before_slot, int after_slot);
 // w -= sum_i coef_i sigma_i V_i, then hout[i] = sigma_i <V_i, w>
 bec_status launch_update_dots(bec_problem* p, double* w,
                               const double* const* V, int nv,
                               const double* sigma, const double* coef,
                               double* hout);
 // out = w + sign sum_i coef_i sigma_i V_i (w may be null = 0, out may be w);
-// if norm_slot >= 0 also scal[norm_slot] = ||out||.
+// norm_slot >= 0: also scal[norm_slot] = ||out||, and with before_slot >= 0 p->flag
+// = (the norm < scal[before_slot] / sqrt(2)): the second Gram-Schmidt pass is needed
+// (the test of Daniel, Gragg, Kaufman and Stewart).  kNormLater: the partials of
+// ||out||^2 are left for launch_arnoldi_end.
+constexpr int kNoNorm = -1, kNormLater = -2;
 bec_status launch_combine(bec_problem* p, double* out, const double* w,
                           const double* const* V, int nv, const double* sigma,
                           const double* coef, double sign, int norm_slot,
-                          const int* flag = nullptr);
-// dots of a finished partial array: hout[i] = sigma_i sum_b partials[i nb + b]
+                          const int* flag = nullptr, int before_slot = -1);
+// dots of a finished partial array: hout[i] = sigma_i sum_b partials[i nb + b];
+// norm_slot >= 0: scal[norm_slot] = sqrt(sum_b partials[nv nb + b])
 bec_status launch_finish_dots(bec_problem* p, int nv, int nb,
                               const double* sigma, double* hout,
-                              const int* flag = nullptr);
-// scal[slot] = ||x||
-bec_status launch_norm(bec_problem* p, const double* x, int slot);
-// Hessenberg column j: H(0:j, j) = h1 + h2 (the two Gram-Schmidt passes),
-// H(j+1, j) = scal[norm_slot] and sigma[j+1] = 1 / H(j+1, j); applies the
-// previous rotations, makes rotation j, updates g and writes |g[j+1]| to
-// scal[res_slot].
-bec_status launch_hessenberg(bec_problem* p, int j, const double* h1,
-                             const double* h2, int norm_slot, int res_slot,
-                             double shift = 0.0);
+                              const int* flag = nullptr, int norm_slot = -1);
+// scal[slot] = ||x||; to_host: also the kScalSlots scalars to the mapped host
+// mirror, by the kernel: a copy could queue behind a large one on a copy engine
+bec_status launch_norm(bec_problem* p, const double* x, int slot, bool to_host);
+// The end of iteration j: scal[norm_slot] = ||v_{j+1}|| from the partials that
+// launch_combine left (not if flag && !*flag); Hessenberg column j: H(0:j, j) =
+// h1 + h2 (the two Gram-Schmidt passes) + shift e_j, H(j+1, j) = scal[norm_slot]
+// and sigma[j+1] = 1 / H(j+1, j); applies the previous rotations, makes rotation
+// j, updates g and writes |g[j+1]| to scal[res_slot]; the scalars to the host.
+bec_status launch_arnoldi_end(bec_problem* p, int j, const double* h1, const double* h2,
+                              int norm_slot, int res_slot, double shift, const int* flag);
 // g = (scal[slot], 0, ...), sigma[0] = 1 / scal[slot].
 bec_status launch_gmres_start(bec_problem* p, int slot);
 // ycoef = H(0:k,0:k)^{-1} g(0:k)
 bec_status launch_least_squares(bec_problem* p, int k);
 bec_status launch_copy(bec_problem* p, const double* x, double* y);
-// copies the kScalSlots scalars to the mapped host mirror with a kernel, so
-// that the read never queues behind a large copy on a copy engine
-bec_status launch_publish_scalars(bec_problem* p);
 bec_status launch_zero(bec_problem* p, double* x);
 
 }  // namespace bec

@@ -155,84 +155,128 @@ sumsq_kernel(const double* __restrict__ x, long long U, double* __restrict__ par
   block_store_sum(nrm, partials);
 }
 
-// hout[v] = sigma_v * sum_b partials[v * nb + b]   (block v, fixed tree order)
+// What follows the passes over the vectors is a handful of numbers: these
+// kernels are bound by their launches and by latency (5 to 7 us each, as long as
+// a pass over 64 x 63 unknowns), so there are few of them: every sum of one
+// pass in one launch, and the norm, the Hessenberg column and the copy to the
+// host in one (8 launches an iteration beside P_eps^{-1} where there were 12).
+
+// sum over the block's threads, on thread 0: pairs (i, i + 128), (i, i + 64), ...
+__device__ __forceinline__ double block_tree_sum(double a) {
+  __shared__ double s[kThreads];
+  s[threadIdx.x] = a;
+  __syncthreads();
+  if (threadIdx.x < 128) s[threadIdx.x] += s[threadIdx.x + 128];
+  __syncthreads();
+  double r = 0.0;
+  if (threadIdx.x < 32)
+    r = warp_sum((s[threadIdx.x] + s[threadIdx.x + 64]) + (s[threadIdx.x + 32] + s[threadIdx.x + 96]));
+  return r;
+}
+
+__device__ __forceinline__ double partials_sum(const double* __restrict__ partials, int nb) {
+  double a = 0.0;
+  for (int b = threadIdx.x; b < nb; b += kThreads) a += partials[b];
+  return block_tree_sum(a);
+}
+
+// the block's scalars, just written by its thread 0, to the host's copy
+__device__ __forceinline__ void publish(const double* scal, double* host) {
+  __syncthreads();
+  if ((int)threadIdx.x < kScalSlots) host[threadIdx.x] = scal[threadIdx.x];
+}
+
+// hout[v] = sigma_v * sum_b partials[v * nb + b]   (block v < nv, fixed tree
+// order); block nv, if launched: scal[norm_slot] = sqrt(sum_b partials[nv * nb + b])
 __global__ void __launch_bounds__(kThreads)
-finish_dots_kernel(const double* __restrict__ partials, int nb, const double* __restrict__ sigma,
-                   double* __restrict__ hout, const int* __restrict__ flag) {
+finish_dots_kernel(const double* __restrict__ partials, int nb, int nv, const double* __restrict__ sigma,
+                   double* __restrict__ hout, const int* __restrict__ flag, double* __restrict__ scal,
+                   int norm_slot) {
   if (flag && *flag == 0) {
     if (threadIdx.x == 0) hout[blockIdx.x] = 0.0;
     return;
   }
-  __shared__ double s[kThreads];
-  double a = 0.0;
-  for (int b = threadIdx.x; b < nb; b += kThreads) a += partials[(long long)blockIdx.x * nb + b];
-  s[threadIdx.x] = a;
-  __syncthreads();
-  for (int st = kThreads / 2; st > 0; st >>= 1) {
-    if ((int)threadIdx.x < st) s[threadIdx.x] += s[threadIdx.x + st];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) hout[blockIdx.x] = s[0] * (sigma ? sigma[blockIdx.x] : 1.0);
+  const double t = partials_sum(partials + (long long)blockIdx.x * nb, nb);
+  if (threadIdx.x != 0) return;
+  if ((int)blockIdx.x == nv) scal[norm_slot] = sqrt(t);
+  else hout[blockIdx.x] = t * (sigma ? sigma[blockIdx.x] : 1.0);
 }
 
-// scal[slot] = sqrt(sum partials)
+// scal[slot] = sqrt(sum partials).  before >= 0: *again = the norm fell below
+// scal[before] / sqrt(2).  host != null: all scalars to the host's copy.
 __global__ void __launch_bounds__(kThreads)
-finish_sqrt_kernel(const double* __restrict__ partials, int nb, double* __restrict__ scal,
-                   int slot, const int* __restrict__ flag) {
-  if (flag && *flag == 0) return;
-  __shared__ double s[kThreads];
-  double a = 0.0;
-  for (int b = threadIdx.x; b < nb; b += kThreads) a += partials[b];
-  s[threadIdx.x] = a;
-  __syncthreads();
-  for (int st = kThreads / 2; st > 0; st >>= 1) {
-    if ((int)threadIdx.x < st) s[threadIdx.x] += s[threadIdx.x + st];
-    __syncthreads();
+finish_sqrt_kernel(const double* __restrict__ partials, int nb, double* scal, int slot, int before,
+                   int* __restrict__ again, double* host) {
+  const double t = partials_sum(partials, nb);
+  if (threadIdx.x == 0) {
+    const double r = sqrt(t);
+    scal[slot] = r;
+    if (before >= 0) again[0] = r * r < 0.5 * scal[before] * scal[before];
   }
-  if (threadIdx.x == 0) scal[slot] = sqrt(s[0]);
+  if (host != nullptr) publish(scal, host);
 }
 
-// Column j of the Arnoldi Hessenberg matrix (leading dimension ldh), the
-// Givens rotations that keep it upper triangular, the rotated right-hand side
-// g whose entry j+1 is the GMRES residual norm, and sigma_{j+1}.
-__global__ void hessenberg_kernel(double* __restrict__ H, int ldh, int j,
-                                  const double* __restrict__ h1, const double* __restrict__ h2,
-                                  double* __restrict__ scal, int norm_slot, int res_slot,
-                                  double* __restrict__ cs, double* __restrict__ sn,
-                                  double* __restrict__ g, double* __restrict__ sigma,
-                                  double shift) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// The end of an Arnoldi iteration, in one block: the norm of the new vector from
+// its partials (flag given and 0: it is in scal already), column j of the Hessenberg
+// matrix (leading dimension ldh), the Givens rotations that keep it upper
+// triangular, the rotated right-hand side g whose entry j+1 is the GMRES residual
+// norm, sigma_{j+1}, and the scalars to the host's copy.  The old rotations run
+// on one thread; its operands are brought to shared memory by the block.
+__global__ void __launch_bounds__(kThreads)
+arnoldi_end_kernel(const double* __restrict__ partials, int nb, const int* __restrict__ flag,
+                   double* __restrict__ H, int ldh, int j, const double* __restrict__ h1,
+                   const double* __restrict__ h2, double* scal, int norm_slot, int res_slot,
+                   double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ g,
+                   double* __restrict__ sigma, double shift, double* host) {
+  __shared__ double sc[kThreads], ss[kThreads], sh[kThreads];
+  double hn = 0.0;                      // thread 0
+  if (flag == nullptr || *flag != 0) {
+    const double t = partials_sum(partials, nb);
+    if (threadIdx.x == 0) scal[norm_slot] = hn = sqrt(t);
+  } else if (threadIdx.x == 0) {
+    hn = scal[norm_slot];
+  }
   double* col = H + (long long)j * ldh;
-  for (int i = 0; i <= j; ++i) col[i] = h1[i] + h2[i];
-  col[j] += shift;   // Arnoldi on (A - shift I): H(A) = H(A - shift I) + shift I
-  const double hn = scal[norm_slot];
-  col[j + 1] = hn;
-  sigma[j + 1] = hn > 0.0 ? 1.0 / hn : 0.0;
-  for (int i = 0; i < j; ++i) {
-    const double a = col[i], b = col[i + 1];
-    col[i] = cs[i] * a + sn[i] * b;
-    col[i + 1] = -sn[i] * a + cs[i] * b;
+  // column entry i before the rotations (Arnoldi on A - shift I: H(A) =
+  // H(A - shift I) + shift I)
+  auto entry = [&](int i) {
+    double h = h1[i] + h2[i];
+    if (i == j) h += shift;
+    return h;
+  };
+  const int i = (int)threadIdx.x;       // j <= kMaxRestart < kThreads
+  if (i < j) {
+    sc[i] = cs[i];
+    ss[i] = sn[i];
+    sh[i] = entry(i + 1);
   }
-  const double a = col[j], b = col[j + 1];
-  double c = 1.0, s = 0.0;
-  if (b != 0.0) {
-    const double r = hypot(a, b);
-    c = a / r;
-    s = b / r;
+  __syncthreads();
+  if (i == 0) {
+    double a = entry(0);                // the entry that the next rotation takes
+    for (int q = 0; q < j; ++q) {
+      const double b = sh[q];
+      sh[q] = sc[q] * a + ss[q] * b;
+      a = -ss[q] * a + sc[q] * b;
+    }
+    const double b = hn;
+    sigma[j + 1] = b > 0.0 ? 1.0 / b : 0.0;
+    double c = 1.0, s = 0.0;
+    if (b != 0.0) {
+      const double r = hypot(a, b);
+      c = a / r;
+      s = b / r;
+    }
+    cs[j] = c;
+    sn[j] = s;
+    col[j] = c * a + s * b;
+    col[j + 1] = 0.0;
+    const double gj = g[j];
+    g[j] = c * gj;
+    g[j + 1] = -s * gj;
+    scal[res_slot] = fabs(g[j + 1]);
   }
-  cs[j] = c;
-  sn[j] = s;
-  col[j] = c * a + s * b;
-  col[j + 1] = 0.0;
-  const double gj = g[j];
-  g[j] = c * gj;
-  g[j + 1] = -s * gj;
-  scal[res_slot] = fabs(g[j + 1]);
-}
-
-__global__ void reorth_flag_kernel(const double* __restrict__ scal, int before, int after,
-                                   int* __restrict__ flag) {
-  if (threadIdx.x == 0) flag[0] = scal[after] * scal[after] < 0.5 * scal[before] * scal[before];
+  publish(scal, host);
+  if (i < j) col[i] = sh[i];
 }
 
 __global__ void gmres_start_kernel(double* __restrict__ g, int len, const double* __restrict__ scal,
@@ -263,11 +307,6 @@ VecList pack(const double* const* V, int n) {
   X(17) X(18) X(19) X(20) X(21) X(22) X(23) X(24) X(25) X(26) X(27) X(28) X(29) X(30)   \
   X(31) X(32)
 
-__global__ void publish_scalars_kernel(const double* __restrict__ scal, double* __restrict__ host,
-                                       int n) {
-  if ((int)threadIdx.x < n) host[threadIdx.x] = scal[threadIdx.x];
-}
-
 bec_status launch_dots_chunk(bec_problem* p, const double* w, VecList L, int n, const int* flag) {
   BEC_LAUNCH_BEGIN(p);
   switch (n) {
@@ -284,27 +323,24 @@ bec_status launch_dots_chunk(bec_problem* p, const double* w, VecList L, int n, 
 }  // namespace
 
 bec_status launch_finish_dots(bec_problem* p, int nv, int nb, const double* sigma, double* hout,
-                              const int* flag) {
+                              const int* flag, int norm_slot) {
   BEC_LAUNCH_BEGIN(p);
-  finish_dots_kernel<<<nv, kThreads, 0, p->stream>>>(p->partials, nb, sigma, hout, flag);
+  finish_dots_kernel<<<nv + (norm_slot >= 0), kThreads, 0, p->stream>>>(p->partials, nb, nv, sigma, hout,
+                                                                        flag, p->scal, norm_slot);
   BEC_LAUNCH_CHECK(p, "finish_dots_kernel");
   return BEC_OK;
 }
 
-bec_status launch_finish_sqrt(bec_problem* p, const double* parts, int nb, int slot,
-                              const int* flag) {
+namespace {
+// scal[slot] = sqrt(sum of the kReduceBlocks partials); see finish_sqrt_kernel
+bec_status launch_finish_sqrt(bec_problem* p, int slot, int before, bool to_host) {
   BEC_LAUNCH_BEGIN(p);
-  finish_sqrt_kernel<<<1, kThreads, 0, p->stream>>>(parts, nb, p->scal, slot, flag);
+  finish_sqrt_kernel<<<1, kThreads, 0, p->stream>>>(p->partials, kReduceBlocks, p->scal, slot, before, p->flag,
+                                                    to_host ? p->host_scal_dev : nullptr);
   BEC_LAUNCH_CHECK(p, "finish_sqrt_kernel");
   return BEC_OK;
 }
-
-bec_status launch_reorth_flag(bec_problem* p, int before_slot, int after_slot) {
-  BEC_LAUNCH_BEGIN(p);
-  reorth_flag_kernel<<<1, 32, 0, p->stream>>>(p->scal, before_slot, after_slot, p->flag);
-  BEC_LAUNCH_CHECK(p, "reorth_flag_kernel");
-  return BEC_OK;
-}
+}  // namespace
 
 bec_status launch_dots(bec_problem* p, const double* w, const double* const* V, int nv,
                        const double* sigma, double* hout, const int* flag) {
@@ -321,7 +357,7 @@ bec_status launch_dots(bec_problem* p, const double* w, const double* const* V, 
 bec_status launch_update_dots(bec_problem* p, double* w, const double* const* V, int nv,
                               const double* sigma, const double* coef, double* hout) {
   if (nv > kMaxVec) {   // unfused: update with every vector, then the dots in chunks
-    bec_status s = launch_combine(p, w, w, V, nv, sigma, coef, -1.0, -1);
+    bec_status s = launch_combine(p, w, w, V, nv, sigma, coef, -1.0, kNoNorm);
     if (s != BEC_OK) return s;
     return launch_dots(p, w, V, nv, sigma, hout);
   }
@@ -343,13 +379,13 @@ bec_status launch_update_dots(bec_problem* p, double* w, const double* const* V,
 
 bec_status launch_combine(bec_problem* p, double* out, const double* w, const double* const* V,
                           int nv, const double* sigma, const double* coef, double sign,
-                          int norm_slot, const int* flag) {
+                          int norm_slot, const int* flag, int before_slot) {
   // chunks of kMaxVec vectors; the norm comes from the last chunk
   int v0 = 0;
   do {
     const int n = nv - v0 < kMaxVec ? nv - v0 : kMaxVec;
     const bool last = v0 + kMaxVec >= nv;
-    double* part = (last && norm_slot >= 0) ? p->partials : nullptr;
+    double* part = (last && norm_slot != kNoNorm) ? p->partials : nullptr;
     const double* src = v0 == 0 ? w : out;
     BEC_LAUNCH_BEGIN(p);
     (part != nullptr ? combine_kernel<true> : combine_kernel<false>)<<<kReduceBlocks, kThreads, 0, p->stream>>>(
@@ -358,24 +394,24 @@ bec_status launch_combine(bec_problem* p, double* out, const double* w, const do
     BEC_LAUNCH_CHECK(p, "combine_kernel");
     v0 += kMaxVec;
   } while (v0 < nv);
-  if (norm_slot >= 0) return launch_finish_sqrt(p, p->partials, kReduceBlocks, norm_slot, flag);
+  if (norm_slot >= 0) return launch_finish_sqrt(p, norm_slot, before_slot, false);
   return BEC_OK;
 }
 
-bec_status launch_norm(bec_problem* p, const double* x, int slot) {
+bec_status launch_norm(bec_problem* p, const double* x, int slot, bool to_host) {
   BEC_LAUNCH_BEGIN(p);
   sumsq_kernel<<<kReduceBlocks, kThreads, 0, p->stream>>>(x, p->U, p->partials);
   BEC_LAUNCH_CHECK(p, "sumsq_kernel");
-  return launch_finish_sqrt(p, p->partials, kReduceBlocks, slot, nullptr);
+  return launch_finish_sqrt(p, slot, -1, to_host);
 }
 
-bec_status launch_hessenberg(bec_problem* p, int j, const double* h1, const double* h2,
-                             int norm_slot, int res_slot, double shift) {
+bec_status launch_arnoldi_end(bec_problem* p, int j, const double* h1, const double* h2, int norm_slot,
+                              int res_slot, double shift, const int* flag) {
   BEC_LAUNCH_BEGIN(p);
-  hessenberg_kernel<<<1, 32, 0, p->stream>>>(p->H, p->max_restart + 1, j, h1, h2, p->scal,
-                                             norm_slot, res_slot, p->cs, p->sn, p->g, p->sigma,
-                                             shift);
-  BEC_LAUNCH_CHECK(p, "hessenberg_kernel");
+  arnoldi_end_kernel<<<1, kThreads, 0, p->stream>>>(p->partials, kReduceBlocks, flag, p->H, p->max_restart + 1,
+                                                    j, h1, h2, p->scal, norm_slot, res_slot, p->cs, p->sn, p->g,
+                                                    p->sigma, shift, p->host_scal_dev);
+  BEC_LAUNCH_CHECK(p, "arnoldi_end_kernel");
   return BEC_OK;
 }
 
@@ -390,13 +426,6 @@ bec_status launch_least_squares(bec_problem* p, int k) {
   BEC_LAUNCH_BEGIN(p);
   least_squares_kernel<<<1, 32, 0, p->stream>>>(p->H, p->max_restart + 1, k, p->g, p->ycoef);
   BEC_LAUNCH_CHECK(p, "least_squares_kernel");
-  return BEC_OK;
-}
-
-bec_status launch_publish_scalars(bec_problem* p) {
-  BEC_LAUNCH_BEGIN(p);
-  publish_scalars_kernel<<<1, 32, 0, p->stream>>>(p->scal, p->host_scal_dev, kScalSlots);
-  BEC_LAUNCH_CHECK(p, "publish_scalars_kernel");
   return BEC_OK;
 }
 

@@ -372,9 +372,9 @@ residual_norms_kernel(const double* __restrict__ f, const double* __restrict__ u
   }
 }
 
-// fslot >= 0: ||f|| is scal[fslot] already
+// fslot >= 0: ||f|| is scal[fslot] already; host != null: the scalars to the host's copy
 __global__ void finish_norms_kernel(const double* __restrict__ partials, long long nblk,
-                                    double* __restrict__ scal, int slot, int fslot) {
+                                    double* scal, int slot, int fslot, double* host) {
   __shared__ double s_a[256], s_b[256];
   double a = 0.0, b = 0.0;
   for (long long i = threadIdx.x; i < nblk; i += blockDim.x) {
@@ -394,6 +394,10 @@ __global__ void finish_norms_kernel(const double* __restrict__ partials, long lo
   if (threadIdx.x == 0) {
     scal[slot] = sqrt(s_a[0]);
     scal[slot + 1] = fslot >= 0 ? scal[fslot] : sqrt(s_b[0]);
+  }
+  if (host != nullptr) {
+    __syncthreads();
+    if ((int)threadIdx.x < kScalSlots) host[threadIdx.x] = scal[threadIdx.x];
   }
 }
 
@@ -891,12 +895,7 @@ bec_status launch_stencil_dots(bec_problem* p, const double* z, double* w,
   }
   BEC_LAUNCH_CHECK(p, "stencil_dots_kernel");
   }
-  bec_status s = BEC_OK;
-  if (norm_slot >= 0) {
-    s = launch_finish_sqrt(p, p->partials + (long long)n * nb, nb, norm_slot, nullptr);
-    if (s != BEC_OK) return s;
-  }
-  s = launch_finish_dots(p, n, nb, sigma, hout);
+  const bec_status s = launch_finish_dots(p, n, nb, sigma, hout, nullptr, norm_slot);
   if (s != BEC_OK || nv <= most) return s;
   // more vectors than one fused launch holds: the rest as plain dots
   return launch_dots(p, w, V + most, nv - most, sigma ? sigma + most : nullptr, hout + most);
@@ -921,7 +920,8 @@ bec_status launch_residual(bec_problem* p, const double* f, const double* u, dou
   return BEC_OK;
 }
 
-bec_status launch_residual_norms(bec_problem* p, const double* f, const double* u, int slot, int fslot) {
+bec_status launch_residual_norms(bec_problem* p, const double* f, const double* u, int slot, int fslot,
+                                 bool to_host) {
   const dim3 grid = stencil_grid(p);
   const StencilGeom g = geom(p);
   long long nblk = (long long)grid.x * grid.y;
@@ -944,7 +944,8 @@ bec_status launch_residual_norms(bec_problem* p, const double* f, const double* 
   BEC_LAUNCH_CHECK(p, "residual_norms_kernel");
   }
   BEC_LAUNCH_BEGIN(p);
-  finish_norms_kernel<<<1, 256, 0, p->stream>>>(p->partials, nblk, p->scal, slot, fslot);
+  finish_norms_kernel<<<1, 256, 0, p->stream>>>(p->partials, nblk, p->scal, slot, fslot,
+                                                to_host ? p->host_scal_dev : nullptr);
   BEC_LAUNCH_CHECK(p, "finish_norms_kernel");
   return BEC_OK;
 }
