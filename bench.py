@@ -56,7 +56,11 @@ ALGO = {
     "time_pass16_tma_kernel": {"flops": 5.0 * LOG2T + 8.0},
     "apply_L_kernel": {"flops": 7.0},
 }
-BYTES_PER_UNIT = {"fp64": {"dst_rows_kernel": 16.0, "dst_cols_kernel": 16.0, "time_pass_kernel": 16.0,
+# The fixed-point passes (FP64 form) move 8 bytes in and out as well; the time
+# pass also reads 16 bytes of reciprocals a mode and frequency.  The fixed-point
+# rows of L read z, f or the basis vectors and write w.
+BYTES_PER_UNIT = {"fp64": {"dst_rows_fx_kernel": 16.0, "dst_cols_fx_kernel": 16.0, "time_fx_kernel": 24.0,
+                           "dst_rows_kernel": 16.0, "dst_cols_kernel": 16.0, "time_pass_kernel": 16.0,
                            "apply_L_kernel": 16.0},
                   "fp32": {"dst_rows_kernel": 12.0, "dst_cols_kernel": 8.0, "time_pass_kernel": 8.0,
                            "dst_cols16_tma_kernel": 8.0, "time_pass16_tma_kernel": 8.0,
@@ -66,13 +70,14 @@ BYTES_PER_UNIT = {"fp64": {"dst_rows_kernel": 16.0, "dst_cols_kernel": 16.0, "ti
 # complex words V (8 B in FP32, 16 B in FP64): smoothing from zero reads b and
 # writes x (2V), a smoothing sweep and the residual read x, b and write one
 # array (3V), restriction reads the fine array and writes a quarter (1.25V),
-# prolongation reads a quarter and updates the fine array (2.25V).  The time
+# prolongation reads a quarter and updates the fine array (2.25V).  An ILU step
+# reads b and 1/D (twice), writes and reads its intermediate and writes x (6V).  The time
 # transforms move one real 8-byte word per space-time unknown plus the half
 # spectrum (0.5V per unknown).
 MG_WORDS = {"mg_smooth0_kernel": 2.0, "mg_smooth_kernel": 3.0, "mg_residual_kernel": 3.0,
-            "mg_restrict_kernel": 1.25, "mg_prolong_add_kernel": 2.25}
+            "mg_restrict_kernel": 1.25, "mg_prolong_add_kernel": 2.25, "ilu_sweep_kernel": 6.0}
 MG_FLOPS = {"mg_smooth0_kernel": 14.0, "mg_smooth_kernel": 98.0, "mg_residual_kernel": 84.0,
-            "mg_restrict_kernel": 36.0, "mg_prolong_add_kernel": 10.0}
+            "mg_restrict_kernel": 36.0, "mg_prolong_add_kernel": 10.0, "ilu_sweep_kernel": 128.0}
 # the finest grid (M = I, 5-point K): B x costs 5 neighbour products and one
 # complex product instead of 9 + 9
 MG_FLOPS_L0 = dict(MG_FLOPS, mg_smooth_kernel=48.0, mg_residual_kernel=32.0)
@@ -105,7 +110,7 @@ def net_fwd_flops(m: int) -> float:
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, from one ncu capture
 # of each kernel at this workload (the P_eps^-1 passes of the second of three
-# applies of `bench.py --ncu-case pinv_fp64`; the command is in the committed
+# applies of `bench.py --ncu-case pinv_fp32`; the command is in the committed
 # DRAM-traffic summary under profiles/).  Each entry carries a SHA-256 prefix
 # of the CUDA sources the kernel is built from, taken when the counters were
 # read: if those sources have changed since, the figure no longer describes
@@ -119,9 +124,6 @@ KERNEL_SOURCES = {
     "time_pass16_tma_kernel": ("bec_time.cu", "bec_passes.cuh", "bec_fft.cuh", "bec_tma.cuh"),
 }
 NCU_TRAFFIC = {
-    ("dst_rows_kernel", "fp64"): (133330688 + 80688896, "d8db73df32f0a703"),
-    ("dst_cols_kernel", "fp64"): (133210368 + 73859840, "d8db73df32f0a703"),
-    ("time_pass_kernel", "fp64"): (200675328 + 75272448, "c598ed99a222731c"),
     ("dst_rows_kernel", "fp32"): (133208320 + 34398464, "d8db73df32f0a703"),
     ("dst_cols16_tma_kernel", "fp32"): (66874624 + 4049920, "99e057cadaa803e3"),
     ("time_pass16_tma_kernel", "fp32"): (66894336 + 4122880, "dac5a038203bb35d"),
@@ -129,10 +131,6 @@ NCU_TRAFFIC = {
 # DRAM bytes of one whole P_eps^-1 apply (the five passes of the same
 # capture) and the kernels whose sources they were taken on
 NCU_PINV_BYTES = {
-    "fp64": ((133330688 + 80688896) + (133210368 + 73859840) + (200675328 + 75272448)
-             + (133211648 + 73844224) + (133211648 + 70523136),
-             {"dst_rows_kernel": "d8db73df32f0a703", "dst_cols_kernel": "d8db73df32f0a703",
-              "time_pass_kernel": "c598ed99a222731c"}),
     "fp32": ((133208320 + 34398464) + (66874624 + 4049920) + (66894336 + 4122880)
              + (66874880 + 3893248) + (66878720 + 69490944),
              {"dst_rows_kernel": "d8db73df32f0a703", "dst_cols16_tma_kernel": "99e057cadaa803e3",
@@ -167,8 +165,9 @@ def ncu_pinv_bytes(form: str):
 
 
 # Algorithmic bytes per unit of one P_eps^-1 apply with five streaming passes:
-# FP64 16 B per pass; FP32 8 B (x-DST in and out: 12 B, one side FP64).
-PINV_BYTES_PER_UNIT = {"fp64": 80.0, "fp32": 48.0}
+# FP64 16 B per pass and 8 B of the time pass's table; FP32 8 B (x-DST in and
+# out: 12 B, one side FP64).
+PINV_BYTES_PER_UNIT = {"fp64": 88.0, "fp32": 48.0}
 
 
 def parse():
@@ -569,7 +568,9 @@ def roofline(form, kernels, U, iters=2):
                 "peak_source": "FP64 FMA units x clock (2/clk/SM x 152 SMs x 2.07 GHz)",
                 "algorithmic_per_unit": f"{ALGO[dom]['flops']:.1f} flop", "units_per_launch": U}
     if dom != "stencil_dots_kernel" and not (form == "fp64" and dom in ALGO):
-        bpu = BYTES_PER_UNIT[form].get(dom, 16.0)
+        # fixed-point rows: z and the j + 1 basis vectors of iteration j in, w out
+        bpu = (16.0 + 8.0 * (iters + 1) / 2.0 if dom == "stencil_dots_fx_kernel" else
+               BYTES_PER_UNIT[form].get(dom, 16.0))
         achieved = bpu * U / (avg_ms / 1e3) / 1e9
         roof = {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": peaks["hbm_gbs"],
                 "unit": "GB/s", "frac": achieved / peaks["hbm_gbs"], "peak_source": peak_src,
@@ -577,7 +578,7 @@ def roofline(form, kernels, U, iters=2):
     roof["avg_launch_ms"] = avg_ms
     roof["traffic"] = ncu_traffic(dom, form)
     roof["traffic_source"] = ("dram__bytes_read.sum + dram__bytes_write.sum of one launch, ncu capture "
-                              "of bench.py --ncu-case pinv_fp64 on the kernel's current sources"
+                              "of bench.py --ncu-case pinv_fp32 on the kernel's current sources"
                               if roof["traffic"] is not None else
                               "no ncu capture of the kernel's current sources")
     return roof
@@ -598,7 +599,7 @@ def pinv_report(form, r, U):
         "peak_source": peak_src, "min_bytes_gbs": round(16.0 * U / t / 1e9, 1),
         "min_bytes_frac": round(16.0 * U / t / 1e9 / peaks["hbm_gbs"], 4),
         "dram_gbs": round(dram / t / 1e9, 1) if dram else None,
-        "bound": "FP64 pipe (2 FMA/clk/SM)" if form == "fp64" else
+        "bound": "integer issue (64-bit fixed-point transforms)" if form == "fp64" else
                  "instruction issue (the FP32 intermediate stays in L2)"}
 
 
@@ -721,7 +722,7 @@ def measure_mg(precision, args, route="mg", train_steps=0, train_batch=16, pre=1
                 "algorithmic_per_unit": "2 x 9 x c_in x c_out FLOP per output pixel and layer",
                 "units_per_launch": "B x side^2 pixels of one layer, B = 2 planes x frequencies",
                 "flops_per_apply": K * net_fwd_flops(m), "avg_launch_ms": avg}
-    elif dom == "stencil_dots_kernel":
+    elif dom in ("stencil_dots_kernel", "stencil_dots_fx_kernel"):
         # the FP64 Krylov operator dominates: bound by the FP64 pipe
         roof = roofline(precision, kernels, U, info["iters"])
     elif base in MG_WORDS:
@@ -734,7 +735,7 @@ def measure_mg(precision, args, route="mg", train_steps=0, train_batch=16, pre=1
     else:
         units = U
         bpu, fpu = 8 + 0.5 * word, 5.0 * LOG2T / 2
-    if route != "learned" and dom != "stencil_dots_kernel":
+    if route != "learned" and dom not in ("stencil_dots_kernel", "stencil_dots_fx_kernel"):
         peaks, src = measured_peaks()
         if precision == "fp64":
             ach = fpu * units / (avg / 1e3) / 1e12

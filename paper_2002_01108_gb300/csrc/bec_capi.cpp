@@ -347,7 +347,10 @@ bec_status bec_allocate_problem(const bec_problem_desc* d, void* stream, bec_pro
   if (s == BEC_OK && d->precision == BEC_PC_FP64 && d->route == BEC_ROUTE_FST &&
       (!fx_wanted(d, t.space.logn, t.time.logn) || fx_setup(p) != BEC_OK))
     chain(dmalloc(&t.rinv64, (size_t)p->J * (N / 2 + 1)));
-  if (s == BEC_OK) mg_alloc_spare(p);   // last: nothing depends on it
+  if (s == BEC_OK) {                    // last: nothing depends on them
+    mg_alloc_spare(p);
+    fx_alloc_spare(p);
+  }
   if (s != BEC_OK) {
     free_all(p);
     delete p;

@@ -509,7 +509,8 @@ struct TimeTile {
     cx v[EPT];
   };
 
-  static BEC_FX void init(Ctx& c, const TimeArgs& g, unsigned char* smem, int tid, long long blk) {
+  // the thread's place in the block's lines; returns the tile's index in its row
+  static BEC_FX int place(Ctx& c, int m, unsigned char* smem, int tid, long long blk) {
     c.tid = tid;
     c.L = tid % LPB;
     c.t = tid / LPB;
@@ -520,13 +521,18 @@ struct TimeTile {
     c.eim = reinterpret_cast<W64*>(smem + kBuf + kStat + kMax);
     c.se = reinterpret_cast<int*>(c.eim + N);
     c.fl = c.se + N;
-    const int XG = (g.m + W) / W;                   // m + 1 = a power of two >= W, or 1
+    const int XG = (m + W) / W;                     // m + 1 = a power of two >= W, or 1
     const long long row = blk / XG;
     const int xg = (int)(blk - row * XG), x0 = xg * W + c.L;
-    c.qa = row * g.m + x0;
+    c.qa = row * m + x0;
     c.qb = c.qa + LPB;
-    c.va = x0 < g.m;
-    c.vb = x0 + LPB < g.m;
+    c.va = x0 < m;
+    c.vb = x0 + LPB < m;
+    return xg;
+  }
+  static BEC_FX void init(Ctx& c, const TimeArgs& g, unsigned char* smem, int tid, long long blk) {
+    const int XG = (g.m + W) / W, xg = place(c, g.m, smem, tid, blk);
+    const long long row = blk / XG;
     const double s = g.scale_dev ? g.scale_dev[0] : 1.0;
     const long long eb = g.dim == 3 ? (row % g.m) * XG + xg : xg;
     const long long es = g.dim == 3 ? (long long)g.m * XG : XG;
@@ -542,7 +548,8 @@ struct TimeTile {
     max_put<THREADS>(c.mx, tid, e);
   }
 
-  static BEC_FX void load(Ctx& c, Reg& r, const TimeArgs& g) {
+  template <typename Args>
+  static BEC_FX void load(Ctx& c, Reg& r, const Args& g) {
     int b0, step;
     bfly_index<LOGN, 0>(c.t, b0, step);
     const i64 *pa = g.data + b0 * g.J + c.qa, *pb = pa + LPB;
@@ -620,12 +627,13 @@ struct TimeTile {
     c.f = (c.ref > kFxNan / 2 ? kFxNan : c.sc.F) + c.sc.s2 + c.sc.s3;
   }
   static BEC_FX void read0(Ctx& c, Reg& r) { pass_read<LOGN, 0>(r.v, c.line, c.t); }
-  static BEC_FX void pass0(Ctx& c, Reg& r, const TimeArgs& g) {
+  template <typename Args>
+  static BEC_FX void pass0(Ctx& c, Reg& r, const Args& g) {
     pass_compute<LOGN, 0, -1>(r.v, g.tw, c.t, c.sc.s2);
     if constexpr (G::NP > 1) pass_write<LOGN, 0>(r.v, c.line, c.t);
   }
-  template <int P>
-  static BEC_FX void pass(Ctx& c, Reg& r, const TimeArgs& g) {
+  template <int P, typename Args>
+  static BEC_FX void pass(Ctx& c, Reg& r, const Args& g) {
     pass_read<LOGN, P>(r.v, c.line, c.t);
     pass_compute<LOGN, P, -1>(r.v, g.tw, c.t, c.sc.s3);
     if constexpr (P + 1 < G::NP) pass_write<LOGN, P>(r.v, c.line, c.t);
@@ -711,6 +719,177 @@ struct TimeTile {
       if (c.vb) pb[j * g.J] = mul64(shr(r.v[i].x + rnd, d), w);
     }
     if (c.tid == 0) g.eout[c.tile] = fm + 1 + g.qe[c.tile];
+  }
+};
+
+// ------------------------------------------- time transforms of the multigrid route
+struct SpecArgs {
+  i64* data;                   // [N][J] FP64 bit patterns
+  double2* spec;               // [N/2+1][J] half spectrum
+  long long J;
+  int m;
+  const double* w;             // eps^{j/N}, inverse: eps^{-j/N}
+  double scale;
+  const double* scale_dev;     // null: 1
+  const CW64* tw;
+};
+
+// The time pass cut open (FP64 in and out): Step 1 to the half spectrum, and
+// Step 3 from one.  A line's unit comes from its largest value alone, so lines
+// of different size in a tile do not lose bits to each other.
+template <int LOGN, int LPB>
+struct SpecTile : TimeTile<LOGN, LPB> {
+  using B = TimeTile<LOGN, LPB>;
+  using typename B::Ctx;
+  using typename B::Reg;
+  using G = Line<LOGN>;
+  using Join = LineJoin<LPB, G::TPL, false>;
+  static constexpr int N = G::n, TPL = G::TPL, EPT = G::EPT, H = EPT / 2, THREADS = B::THREADS;
+  static constexpr int R1 = B::R1, RL = B::RL;
+
+  static BEC_FX double to_d(i64 v, int f) {
+    return fx_normal(f) ? fx_to_d(v, f) : f > kFxNan / 2 ? bits_d(0x7FF8000000000000ULL) : fx_to_d_slow(v, f);
+  }
+  static BEC_FX void init(Ctx& c, const SpecArgs& g, unsigned char* smem, int tid, long long blk) {
+    B::place(c, g.m, smem, tid, blk);
+    const double s = g.scale_dev ? g.scale * g.scale_dev[0] : g.scale;
+    int e = -kFxNan;
+    for (int j = tid; j < N; j += THREADS) {
+      int x;
+      c.eim[j] = mant_of(g.w[j] * s, x);
+      c.se[j] = x;
+      e = e > x ? e : x;
+    }
+    max_put<THREADS>(c.mx, tid, e);
+  }
+  // the largest exponent field of the line, in two phases; the lines' shared
+  // memory is free until the first pass
+  static BEC_FX Stat* scratch(const Ctx& c) { return reinterpret_cast<Stat*>(c.line - c.L * G::STRIDE); }
+  static BEC_FX void max_in(Ctx& c, const Reg& r) {
+    int h = 0;
+#pragma unroll
+    for (int i = 0; i < EPT; ++i) {
+      const int x = d_habs((u64)r.v[i].x), y = d_habs((u64)r.v[i].y), w = x > y ? x : y;
+      h = h > w ? h : w;
+    }
+    c.s = {(float)(h >> 20), 0.f};
+    Join::put(scratch(c), c.s, c.tid, c.L);
+  }
+  // the line's values as integers below 2^bits; returns their exponent
+  static BEC_FX int to_fixed(Ctx& c, Reg& r, int bits) {
+    const int em = (int)Join::get(scratch(c), c.s, c.tid, c.L).m;
+    int f = em - 1022 - bits;
+    if (f < kFxMin) f = kFxMin;
+#pragma unroll
+    for (int i = 0; i < EPT; ++i) r.v[i] = cx{d_to_fx((u64)r.v[i].x, f), d_to_fx((u64)r.v[i].y, f)};
+    c.f = em == 0x7FF ? kFxNan : 0;
+    return f;
+  }
+
+  // forward: values, then the statistics as in TimeTile::measure
+  static BEC_FX void measure(Ctx& c, Reg& r) {
+    c.ref = to_fixed(c, r, 62);
+    const int e = max_get<THREADS>(c.mx);
+    int b0, step;
+    bfly_index<LOGN, 0>(c.t, b0, step);
+    float m = 0.f, la = 0.f, lb = 0.f;
+#pragma unroll
+    for (int i = 0; i < EPT; ++i) {
+      int bu, st;
+      bfly_index<LOGN, 0>(TPL * (i / R1), bu, st);
+      const int d = e - c.se[b0 + bu + (i % R1) * st];
+      const float x = mag(r.v[i].x, d), y = mag(r.v[i].y, d);
+      m = fmaxf(m, fmaxf(x, y));
+      la += x;
+      lb += y;
+    }
+    c.s = {m, fmaxf(la, lb)};
+    Join::put(c.st, c.s, c.tid, c.L);
+  }
+  static BEC_FX void first(Ctx& c, Reg& r) {
+    const Stat s = Join::get(c.st, c.s, c.tid, c.L);
+    const int e = max_get<THREADS>(c.mx);
+    c.sc = line_scale<LOGN>(c.ref + e, (float)R1 * 1.4143f * (s.m + 1.f), 2.f * (s.l + (float)N));
+    const int fi = c.sc.F - 1;                      // w times 2^63: half
+    int b0, step;
+    bfly_index<LOGN, 0>(c.t, b0, step);
+#pragma unroll
+    for (int i = 0; i < EPT; ++i) {
+      int bu, st;
+      bfly_index<LOGN, 0>(TPL * (i / R1), bu, st);
+      const int j = b0 + bu + (i % R1) * st, d = fi - c.ref - c.se[j];
+      const i64 init = d > 0 ? kHalf + kHalf / 2 : kHalf;
+      r.v[i] = cx{mul64(shift(r.v[i].x, d), c.eim[j], init), mul64(shift(r.v[i].y, d), c.eim[j], init)};
+    }
+    if (e > kFxNan / 2) c.f = kFxNan;
+    c.f += (c.f == kFxNan ? 0 : c.sc.F) + c.sc.s2 + c.sc.s3;
+  }
+  // the two lines' spectra at k, separated
+  static BEC_FX void put(const Ctx& c, const SpecArgs& g, int k, cx C, cx Cn) {
+    const int f = c.f - 1;
+    double2* p = g.spec + k * g.J;
+    if (c.va) p[c.qa] = make_double2(to_d(C.x + Cn.x, f), to_d(C.y - Cn.y, f));
+    if (c.vb) p[c.qb] = make_double2(to_d(C.y + Cn.y, f), to_d(Cn.x - C.x, f));
+  }
+  static BEC_FX void store(Ctx& c, const SpecArgs& g) {
+    const cx* fp = c.line + slot(c.t);
+#pragma unroll
+    for (int u = 0; u < H; ++u)
+      put(c, g, c.t + TPL * u, fp[slot(TPL * u)], c.line[slot(u == 0 && c.t == 0 ? 0 : N - c.t - TPL * u)]);
+    if (c.t == 0) put(c, g, N / 2, c.line[slot(N / 2)], c.line[slot(N / 2)]);
+  }
+
+  // inverse: v[2 u], v[2 u + 1] = the two lines' values at k = t + TPL u; of the
+  // real frequencies 0 and N/2 the real parts, side by side
+  static BEC_FX void load_spec(Ctx& c, Reg& r, const SpecArgs& g) {
+    const i64 *pa = reinterpret_cast<const i64*>(g.spec + c.t * g.J + c.qa), *pb = pa + 2 * LPB;
+#pragma unroll
+    for (int i = 0; i < EPT; ++i) r.v[i] = cx{0, 0};
+    if (c.va) {
+#pragma unroll
+      for (int u = 0; u < H; ++u) r.v[2 * u] = cx{pa[2 * TPL * u * g.J], pa[2 * TPL * u * g.J + 1]};
+      if (c.t == 0) r.v[0].y = pa[N * g.J];
+    }
+    if (c.vb) {
+#pragma unroll
+      for (int u = 0; u < H; ++u) r.v[2 * u + 1] = cx{pb[2 * TPL * u * g.J], pb[2 * TPL * u * g.J + 1]};
+      if (c.t == 0) r.v[1].y = pb[N * g.J];
+    }
+  }
+  // A + i B at k and conj(A) + i conj(B) at N - k, and what rescale() wants
+  static BEC_FX void measure_spec(Ctx& c, Reg& r) {
+    const int f = to_fixed(c, r, 61);
+    c.f += c.f == kFxNan ? 0 : f - 1;               // rescale() counts a factor 2
+    float m = 0.f, l = 0.f;
+#pragma unroll
+    for (int u = 0; u < H; ++u) {
+      const cx A = r.v[2 * u], Bv = r.v[2 * u + 1];
+      const bool real = u == 0 && c.t == 0;
+      r.v[2 * u] = real ? cx{A.x, Bv.x} : cx{A.x - Bv.y, A.y + Bv.x};
+      r.v[2 * u + 1] = real ? cx{A.y, Bv.y} : cx{A.x + Bv.y, Bv.x - A.y};
+    }
+#pragma unroll
+    for (int i = 0; i < EPT; ++i) {
+      const float x = mag(r.v[i].x), y = mag(r.v[i].y);
+      m = fmaxf(m, fmaxf(x, y));
+      l += x + y;
+    }
+    c.s = {m, l};
+    Join::put(c.st, c.s, c.tid, c.L);
+  }
+  static BEC_FX void store_time(Ctx& c, Reg& r, const SpecArgs& g) {
+    int b0, step;
+    out_index<LOGN>(c.t, b0, step);
+    double *pa = reinterpret_cast<double*>(g.data) + b0 * g.J + c.qa, *pb = pa + LPB;
+#pragma unroll
+    for (int i = 0; i < EPT; ++i) {
+      int bu, st;
+      out_index<LOGN>(TPL * (i / RL), bu, st);
+      const int j = bu + (i % RL) * st, f = c.f + 1 + c.se[b0 + j];
+      const W64 w = c.eim[b0 + j];                  // half
+      if (c.va) pa[j * g.J] = to_d(mul64(r.v[i].y, w), f);
+      if (c.vb) pb[j * g.J] = to_d(mul64(r.v[i].x, w), f);
+    }
   }
 };
 

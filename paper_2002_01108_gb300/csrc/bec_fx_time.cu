@@ -76,6 +76,74 @@ bec_status fx_time_w(bec_problem* p, const TimeArgs& g) {
   return p->fx.lpb == 8 ? fx_time_launch<LOGN, 8>(p, g) : fx_time_launch<LOGN, 16>(p, g);
 }
 
+// The multigrid route's time transforms (FP64).  The floating-point kernels
+// (bec_time.cu) are bound by the FP64 pipe: at 127^2 x 64 (1M unknowns) 83 us
+// forward and 80 back, where these take 16, a good part of it launch and
+// latency (16.5 MB of traffic are 2.4 us of HBM).
+template <typename Tile, bool INV>
+__global__ void __launch_bounds__(Tile::THREADS, fxt_blocks(Tile::THREADS)) time_spec_fx_kernel(SpecArgs g) {
+  extern __shared__ __align__(16) unsigned char fx_smem[];
+  typename Tile::Ctx c;
+  typename Tile::Reg r;
+  Tile::init(c, g, fx_smem, threadIdx.x, blockIdx.x);
+  if constexpr (INV) Tile::load_spec(c, r, g);
+  else Tile::load(c, r, g);
+  Tile::max_in(c, r);
+  __syncthreads();
+  if constexpr (INV) Tile::measure_spec(c, r);
+  else Tile::measure(c, r);
+  __syncthreads();
+  if constexpr (INV) {
+    Tile::rescale(c, r);
+    __syncthreads();
+    Tile::read0(c, r);
+  } else {
+    Tile::first(c, r);
+  }
+  Tile::pass0(c, r, g);
+  if constexpr (Tile::G::NP > 1) {
+    __syncthreads();
+    Tile::template pass<1>(c, r, g);
+  }
+  if constexpr (Tile::G::NP > 2) {
+    __syncthreads();
+    Tile::template pass<2>(c, r, g);
+  }
+  if constexpr (INV) {
+    Tile::store_time(c, r, g);
+  } else {
+    __syncthreads();
+    Tile::natural(c, r);
+    __syncthreads();
+    Tile::store(c, g);
+  }
+}
+
+template <int LOGN, int LPB, bool INV>
+bec_status fx_spec_launch(bec_problem* p, const SpecArgs& g) {
+  using Tile = SpecTile<LOGN, LPB>;
+  auto k = time_spec_fx_kernel<Tile, INV>;
+  if (Tile::SMEM > 48 * 1024)
+    BEC_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tile::SMEM));
+  BEC_LAUNCH_BEGIN(p);
+  k<<<(unsigned)(p->J / p->m * fx_xg(p)), Tile::THREADS, Tile::SMEM, p->stream>>>(g);
+  BEC_LAUNCH_CHECK(p, INV ? "time_inv_fx_kernel" : "time_fwd_fx_kernel");
+  return BEC_OK;
+}
+template <bool INV>
+bec_status fx_spec(bec_problem* p, const SpecArgs& g) {
+  switch (p->tab.time.logn) {
+    case 5: return fx_spec_launch<5, 16, INV>(p, g);
+    case 6: return fx_spec_launch<6, 16, INV>(p, g);
+    case 7: return fx_spec_launch<7, 16, INV>(p, g);
+    case 8: return fx_spec_launch<8, 16, INV>(p, g);
+    case 9: return fx_spec_launch<9, 8, INV>(p, g);
+    default: break;
+  }
+  set_error("unsupported number of time steps");
+  return BEC_EUNSUPPORTED;
+}
+
 // q[k][q] = scale conj(d) / |d|^2 with d = lambda'_k mu^M + tau mu^K, times
 // 2^(63 - qe): the smallest |d| of the W modes of a tile (W lanes) sets qe so
 // that |q| stays below 0.9.
@@ -222,6 +290,35 @@ bec_status fx_setup(bec_problem* p) {
   t.e0 = ints(o_e0);
   t.e1 = ints(o_e1);
   return BEC_OK;
+}
+
+void fx_alloc_spare(bec_problem* p) {
+  const int logt = p->tab.time.logn;
+  if (p->desc.precision != BEC_PC_FP64 || p->desc.route == BEC_ROUTE_FST || logt < 5 || logt > 9) return;
+  const std::vector<CW64> tt = fx_twiddles(logt);
+  const size_t bytes = tt.size() * sizeof(CW64);
+  FxTables& t = p->fx;
+  if (cudaMalloc(&t.tables, bytes) != cudaSuccess ||
+      cudaMemcpy(t.tables, tt.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
+    fx_free(p);
+    cudaGetLastError();
+    return;
+  }
+  t.tw_time = t.tables;
+  t.lpb = logt >= 9 ? 8 : 16;
+}
+
+bec_status launch_fx_spec(bec_problem* p, const double* y, double* z, void* spec, const double* scale_dev) {
+  SpecArgs g{};
+  g.data = reinterpret_cast<i64*>(y != nullptr ? const_cast<double*>(y) : z);
+  g.spec = static_cast<double2*>(spec);
+  g.J = p->J;
+  g.m = p->m;
+  g.w = y != nullptr ? p->tab.es64 : p->tab.eis64;
+  g.scale = y != nullptr ? 1.0 : 1.0 / p->N;
+  g.scale_dev = scale_dev;
+  g.tw = static_cast<const CW64*>(p->fx.tw_time);
+  return y != nullptr ? fx_spec<false>(p, g) : fx_spec<true>(p, g);
 }
 
 bec_status fx_set_eps(bec_problem* p, const std::vector<double>& es) {

@@ -306,6 +306,11 @@ inline bool fx_applies(const bec_problem* p) { return p->fx.q != nullptr; }
 // out), column DSTs and time pass on integers, in place
 bec_status launch_fx_rows(bec_problem* p, const double* in, double* out, bool forward);
 bec_status launch_fx_cols(bec_problem* p, double* data, bool forward);
+// the multigrid route's time transforms in fixed point (FP64, 32 <= N <= 512): y
+// to the half spectrum, or (y null) the half spectrum to z.  fx_alloc_spare makes
+// their table; without the memory for it the floating-point kernels run
+bec_status launch_fx_spec(bec_problem* p, const double* y, double* z, void* spec, const double* scale_dev);
+void fx_alloc_spare(bec_problem* p);
 bec_status launch_fx_time(bec_problem* p, double* data, const double* scale_dev);
 // rinv64[q][k] = 1 / |lambda'_k + tau mu_q|^2 from the current lambda' table
 bec_status launch_rinv_table(bec_problem* p);

@@ -415,6 +415,7 @@ bec_status time_inv_launch(bec_problem* p, const void* spec, double* z, double s
 bec_status launch_time_fwd(bec_problem* p, const double* y, void* spec, int fp64,
                            const double* scale_dev) {
   const PcTables& t = p->tab;
+  if (fp64 && p->fx.tw_time != nullptr) return launch_fx_spec(p, y, nullptr, spec, scale_dev);
   if (fp64) {
 #define BEC_FWD64(L) time_fwd_launch<double, L>(p, y, spec, 1.0, scale_dev, t.es64, t.time.tw64)
     BEC_TIME_SWITCH(t.time.logn, BEC_FWD64)
@@ -431,6 +432,8 @@ bec_status launch_time_fwd(bec_problem* p, const double* y, void* spec, int fp64
 bec_status launch_time_inv(bec_problem* p, const void* spec, double* z, int fp64) {
   const PcTables& t = p->tab;
   const double scale = 1.0 / p->N;
+  if (fp64 && p->fx.tw_time != nullptr)
+    return launch_fx_spec(p, nullptr, z, const_cast<void*>(spec), nullptr);
   if (fp64) {
 #define BEC_INV64(L) time_inv_launch<double, L>(p, spec, z, scale, t.eis64, t.time.tw64)
     BEC_TIME_SWITCH(t.time.logn, BEC_INV64)
