@@ -451,6 +451,7 @@ constexpr int kFxDotVecs = 8;        // vectors a fused launch takes; more go to
 
 struct FxStencil {
   fx::W64 cm;      // c = cm 2^-63 2^ce
+  fx::W64 wa[3], wm[3];   // Q1: centre, edge, corner of M + tau K and of M, times 2^(63 - ce)
   int ce;
   int chunk;       // time steps of a tile
   int xt, yg, planes;   // tiles in x, row groups, planes (3D: m)
@@ -463,18 +464,20 @@ enum { kModeDots = 0, kModeNorms = 1, kModeApply = 2, kModeResidual = 3 };
 template <int KIND, int P>
 __device__ __noinline__ double fx_slow_row(const double* __restrict__ vs, long long q, int ix, int iy, int iz,
                                            int n, const StencilGeom& g) {
-  return row_of<KIND, P>(vs, nullptr, nullptr, q, ix, iy, iz, g, vs[q], n > 0 ? vs[q - g.J] : 0.0,
+  return row_of<KIND, P>(vs, KIND == kQ1 && n > 0 ? vs - g.J : nullptr, nullptr, q, ix, iy, iz, g, vs[q],
+                         n > 0 ? vs[q - g.J] : 0.0,
                          P == 2 && n > 1 ? vs[q - 2 * g.J] : 0.0);
 }
 
 template <int KIND, int P>
 struct FxRow {
   static constexpr int R = kFxRows;
-  static constexpr bool D3 = KIND == kFD3;
+  static constexpr bool D3 = KIND == kFD3, Q1 = KIND == kQ1;
+  static constexpr int ER = Q1 ? R + 2 : R;   // rows whose left and right ends are wanted
   // one slice's values of the tile, as bit patterns (zeros outside the domain)
   struct Raw {
     fx::u64 b[R + 2];        // the lane's column: the row below, the rows, the row above
-    fx::u64 edge;            // lane r < R: left of row r; lane R + r: right of it
+    fx::u64 edge;            // lane r < ER: left of row r (Q1: r - 1); lane ER + r: right of it
     fx::u64 d[D3 ? R : 1], u[D3 ? R : 1];   // 3D: the planes below and above
   };
   int m, lane, x, y0, z0, rows;
@@ -498,8 +501,9 @@ struct FxRow {
       if (y0 > 0) in |= 1u;
       if (y0 + rows < m) in |= 1u << (rows + 1);
     }
-    const int er = lane % R, ex = lane < R ? x0 - 1 : x0 + 32;
-    if (lane < 2 * R && er < rows && ex >= 0 && ex < m) in |= 1u << 31;
+    const int er = lane % ER - (Q1 ? 1 : 0), ex = lane < ER ? x0 - 1 : x0 + 32;
+    if (lane < 2 * ER && er < rows + (Q1 ? 1 : 0) && y0 + er >= 0 && y0 + er < m && ex >= 0 && ex < m)
+      in |= 1u << 31;
     eo = ((long long)z0 * m + y0 + er) * m + ex;
   }
   __device__ __forceinline__ bool row_in(int r) const { return in >> (r + 1) & 1; }
@@ -530,6 +534,73 @@ struct FxRow {
     F = max(e - 1081, fx::kFxMin);
 #pragma unroll
     for (int r = 0; r < R; ++r) pv[r] = fx::d_to_fx(b[r], F);
+  }
+  // Q1: visit(r, centre, sum of the 4 edge neighbours, of the 4 corners) for the
+  // rows of a slice, in the unit 2^F
+  template <typename Visit>
+  __device__ __forceinline__ void q1_rows(const Raw& w, int F, Visit visit) const {
+    using fx::i64;
+    const i64 edge = fx::d_to_fx(w.edge, F);
+    auto ends = [&](i64 c, int r) {                       // left plus right of row r - 1
+      i64 le = __shfl_up_sync(0xffffffffu, c, 1), ri = __shfl_down_sync(0xffffffffu, c, 1);
+      const i64 ed = __shfl_sync(0xffffffffu, edge, lane < 16 ? r : ER + r);
+      if (lane == 0) le = ed;
+      if (lane == 31) ri = ed;
+      return le + ri;
+    };
+    i64 below = fx::d_to_fx(w.b[0], F), c = fx::d_to_fx(w.b[1], F);
+    i64 hb = ends(below, 0), h = ends(c, 1);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const i64 above = fx::d_to_fx(w.b[r + 2], F), ha = ends(above, r + 2);
+      visit(r, c, h + (below + above), hb + ha);
+      below = c;
+      c = above;
+      hb = h;
+      h = ha;
+    }
+  }
+  __device__ __forceinline__ int q1_max(const Raw& w) const {
+    int h = fx::d_habs(w.edge);
+#pragma unroll
+    for (int r = 0; r < R + 2; ++r) h = max(h, fx::d_habs(w.b[r]));
+    return (int)__reduce_max_sync(0xffffffffu, (unsigned)h) >> 20;
+  }
+  static __device__ __forceinline__ fx::i64 q1_form(const fx::W64 (&k)[3], fx::i64 c, fx::i64 e, fx::i64 d) {
+    return (fx::mul64(c, k[0]) + fx::mul64(e, k[1])) + fx::mul64(d, k[2]);
+  }
+  // prev = M times the slice vs
+  __device__ __forceinline__ void load_prev_q1(const double* __restrict__ vs, const FxStencil& f) {
+    Raw w;
+    if (vs != nullptr) load(vs, w);
+    else w = Raw{};
+    ep = q1_max(w);
+    Fp = max(ep - 1081, fx::kFxMin);
+    q1_rows(w, Fp, [&](int r, fx::i64 c, fx::i64 e, fx::i64 d) { prev[r] = q1_form(f.wm, c, e, d); });
+  }
+  // y = rows of (M + tau K) v^n - M v^{n-1}.  |v| < 2^59 and |coefficient| < 2^63:
+  // each of the two parts stays below 2^61.2
+  __device__ __forceinline__ void step_q1(const Raw& w, const double* __restrict__ vs, const StencilGeom& g,
+                                          const FxStencil& f, int n, double (&y)[R]) {
+    const int e = q1_max(w), em = max(e, ep);
+    const int F = max(em - 1081, fx::kFxMin), G = F + f.ce + 1;
+    if (F != Fp) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) prev[r] = fx::shift(prev[r], F - Fp);
+    }
+    const bool plain = em != 0x7FF && fx::fx_normal(G);
+    q1_rows(w, F, [&](int r, fx::i64 c, fx::i64 eg, fx::i64 d) {
+      const fx::i64 Y = q1_form(f.wa, c, eg, d) - prev[r];
+      prev[r] = q1_form(f.wm, c, eg, d);
+      if (plain) y[r] = fx::fx_to_d(Y, G);
+    });
+    if (!plain) {
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        y[r] = row_in(r) ? fx_slow_row<KIND, P>(vs, q0 + r * m, x, y0 + r, z0, n, g) : 0.0;
+    }
+    ep = e;
+    Fp = F;
   }
   // y = row values of the slice vs = v^n, whose values are in w
   __device__ __forceinline__ void step(const Raw& w, const double* __restrict__ vs, const StencilGeom& g,
@@ -609,7 +680,7 @@ struct FxRow {
 // residual_norms_kernel (aux = f; LAST: without f^2); kModeApply: w = L z (times *sshift if
 // given); kModeResidual: w = aux - L z.
 template <int MODE, int NV, bool LAST, int KIND, int P>
-__global__ void __launch_bounds__(kStencilThreads, NV <= 2 && KIND != kFD3 ? 3 : 2)
+__global__ void __launch_bounds__(kStencilThreads, NV <= 2 && KIND == kFD ? 3 : 2)
 stencil_fx_kernel(const double* __restrict__ z, const double* __restrict__ aux, double* __restrict__ w,
                   StencilGeom g, FxStencil f, VecList V, const double* __restrict__ vshift,
                   const double* __restrict__ sshift, double* __restrict__ partials) {
@@ -629,7 +700,8 @@ stencil_fx_kernel(const double* __restrict__ z, const double* __restrict__ aux, 
     const double* zs = z + (long long)n0 * g.J;
     typename Row::Raw cur, nxt;
     row.load(zs, cur);
-    row.load_prev(n0 > 0 ? zs - g.J : nullptr, row.prev, row.Fp, row.ep);
+    if constexpr (Row::Q1) row.load_prev_q1(n0 > 0 ? zs - g.J : nullptr, f);
+    else row.load_prev(n0 > 0 ? zs - g.J : nullptr, row.prev, row.Fp, row.ep);
     if constexpr (P == 2)
       row.load_prev(n0 > 1 ? zs - 2 * g.J : nullptr, row.prev2, row.Fp2, row.ep2);
     long long o0 = (long long)n0 * g.J + row.q0;
@@ -646,7 +718,8 @@ stencil_fx_kernel(const double* __restrict__ z, const double* __restrict__ aux, 
         else if constexpr (MODE != kModeApply) a1[r] = aux[o0 + r * g.m];
       }
       double y[R];
-      row.step(cur, zs, g, f, n, y);
+      if constexpr (Row::Q1) row.step_q1(cur, zs, g, f, n, y);
+      else row.step(cur, zs, g, f, n, y);
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         if (!row.row_in(r)) continue;
@@ -771,22 +844,35 @@ void stencil_dots_launch(int var, cudaStream_t st, const double* z, double* w,
 #undef BEC_SD_LAUNCH
 }
 
-// The fixed-point rows take finite differences with a constant coefficient in 2D
-// and 3D from 31 points a side (a warp's 32 columns are then nearly full).
+// The fixed-point rows take constant coefficients in 2D and 3D from 31 points a
+// side (a warp's 32 columns are then nearly full): finite differences, and Q1
+// elements (2D) with the one-step scheme.
 bool fx_rows(const bec_problem* p) {
-  return p->kcoef == nullptr && p->desc.space == BEC_SPACE_FD && p->dim >= 2 && p->m >= 31;
+  return p->kcoef == nullptr && p->dim >= 2 && p->m >= 31 &&
+         (p->desc.space == BEC_SPACE_FD || p->desc.time_scheme != BEC_TIME_BDF2);
+}
+
+// w = v 2^(63 - ce), |v| < 2^ce, as two words
+fx::W64 fx_coef(double v, int ce) {
+  long long w = (long long)std::ldexp(v, 63 - ce);
+  if ((int)w == (int)0x80000000) ++w;             // the low word can be negated
+  return fx::split64(w);
 }
 
 // blocks: what the card holds at once (3 a SM), or fewer
 unsigned fx_stencil(const bec_problem* p, const StencilGeom& g, FxStencil& f) {
   int ce;
-  const double cm = std::frexp(g.c, &ce);
-  long long w = (long long)std::ldexp(cm, 63);
-  if (w > 0x7FFFFFFF00000000LL) {                 // next to 1: half of it
-    w >>= 1;
-    ++ce;
+  const bool q1 = p->desc.space == BEC_SPACE_Q1;
+  double top = g.c;
+  if (q1) top = std::max(std::max(std::max(std::fabs(g.ac), std::fabs(g.ae)), std::fabs(g.ak)), g.mc);
+  const double cm = std::frexp(top, &ce);
+  if (cm > 0.9999999) ++ce;                       // next to 1: half of it
+  const double wa[3] = {g.ac, g.ae, g.ak}, wm[3] = {g.mc, g.me, g.mk};
+  for (int i = 0; i < 3; ++i) {
+    f.wa[i] = fx_coef(wa[i], ce);
+    f.wm[i] = fx_coef(wm[i], ce);
   }
-  f.cm = fx::split64(w);
+  f.cm = fx_coef(q1 ? 0.0 : g.c, ce);
   f.ce = ce;
   f.xt = (p->m + 31) / 32;
   f.yg = (p->m + kFxRows - 1) / kFxRows;
@@ -809,6 +895,7 @@ void stencil_fx_launch(const bec_problem* p, unsigned grid, const double* z, con
   stencil_fx_kernel<MODE, NV, LAST, K, P><<<grid, kStencilThreads, 0, p->stream>>>(               \
       z, aux, w, g, f, L, vshift, sshift, p->partials)
   if (p->dim == 3) BEC_SFX(kFD3, 1);
+  else if (p->desc.space == BEC_SPACE_Q1) BEC_SFX(kQ1, 1);
   else if (p->desc.time_scheme == BEC_TIME_BDF2) BEC_SFX(kFD, 2);
   else BEC_SFX(kFD, 1);
 #undef BEC_SFX
