@@ -108,7 +108,6 @@ __device__ __forceinline__ double mass_row_q1(const double* __restrict__ us, lon
 // The operator a kernel instantiation applies: finite differences in 1D or
 // 2D (constant or variable a), Q1 elements (1D or 2D), finite differences in 3D.
 enum { kFD = 0, kQ1 = 1, kFD3 = 2 };
-constexpr int kFDV = 3;   // of the fixed-point rows: finite differences with variable coefficients
 
 // point q of a slice as (ix, iy, iz): x fastest, rows of m points
 template <int KIND>
@@ -428,8 +427,8 @@ __global__ void build_rhs_kernel(const double* __restrict__ u0, const double* __
 }
 
 // ---------------------------------------------------------------- fixed point
-// The rows of L in 64-bit fixed point (bec_fx.cuh): finite differences in 2D (also
-// with variable coefficients) and 3D, Q1 elements in 2D.
+// The finite-difference rows of L in 64-bit fixed point (bec_fx.cuh), 2D and
+// 3D with a constant coefficient.
 //
 // GB300 issues 2 FP64 operations a clock and SM: the 5 (2D) or 7 (3D) of a row
 // bound the kernels above, whose vectors' traffic takes a quarter of that time.
@@ -447,15 +446,6 @@ __global__ void build_rhs_kernel(const double* __restrict__ u0, const double* __
 // Measured at 255^2 x 256: w = L z - s v with 1 and 2 dots 161 us on average
 // (FP64 rows: 287), ||f - L u|| 116 us (300); what bounds them now is the FP64
 // pipe again (2 operations and one a dot), 70 to 80 % busy.
-//
-// Q1 rows take six products, three of them by M, which the next step's row
-// subtracts: a lane keeps M v^{n-1} instead of the values.  At 127^2 x 64 (1M
-// unknowns) L v takes 20 us (FP64 rows: 56), ||f - L u|| 24 us (61).
-//
-// Variable coefficients take five products a row; a lane brings the
-// coefficients of its rows to fixed point once a tile and keeps them in shared
-// memory.  At 255^2 x 256 w with 1 to 8 dots takes 340 us on average (390), the
-// residual 204 us (309): the dots bound it.
 constexpr int kFxRows = 4;
 constexpr int kFxDotVecs = 8;        // vectors a fused launch takes; more go to dots_kernel
 
@@ -474,7 +464,7 @@ enum { kModeDots = 0, kModeNorms = 1, kModeApply = 2, kModeResidual = 3 };
 template <int KIND, int P>
 __device__ __noinline__ double fx_slow_row(const double* __restrict__ vs, long long q, int ix, int iy, int iz,
                                            int n, const StencilGeom& g) {
-  return row_of<KIND == kFDV ? kFD : KIND, P>(vs, KIND == kQ1 && n > 0 ? vs - g.J : nullptr, nullptr, q, ix, iy, iz, g, vs[q],
+  return row_of<KIND, P>(vs, KIND == kQ1 && n > 0 ? vs - g.J : nullptr, nullptr, q, ix, iy, iz, g, vs[q],
                          n > 0 ? vs[q - g.J] : 0.0,
                          P == 2 && n > 1 ? vs[q - 2 * g.J] : 0.0);
 }
@@ -482,7 +472,7 @@ __device__ __noinline__ double fx_slow_row(const double* __restrict__ vs, long l
 template <int KIND, int P>
 struct FxRow {
   static constexpr int R = kFxRows;
-  static constexpr bool D3 = KIND == kFD3, Q1 = KIND == kQ1, VAR = KIND == kFDV;
+  static constexpr bool D3 = KIND == kFD3, Q1 = KIND == kQ1;
   static constexpr int ER = Q1 ? R + 2 : R;   // rows whose left and right ends are wanted
   // one slice's values of the tile, as bit patterns (zeros outside the domain)
   struct Raw {
@@ -494,8 +484,6 @@ struct FxRow {
   unsigned in;               // which of b[] lie inside the domain; bit 31: the edge value
   long long q0, eo;          // the lane's first row; its edge value's point
   fx::i64 prev[R], prev2[P == 2 ? R : 1];
-  static constexpr int kNoScale = 1 << 28;   // coefficients that are not finite
-  int cs;                    // VAR: coefficient times 2^(64 - cs) is stored
   int Fp, Fp2, ep, ep2;      // unit and largest exponent field of prev, prev2
 
   __device__ __forceinline__ void start(const StencilGeom& g, const FxStencil& f, int t, int ln) {
@@ -614,68 +602,6 @@ struct FxRow {
     ep = e;
     Fp = F;
   }
-  // VAR: the lane's coefficients [centre, W, E, S, N] of its rows to its column
-  // of cf, times 2^-(cs - 64): one power of two for the warp's tile, so that a
-  // large coefficient elsewhere costs no bits here
-  __device__ __forceinline__ void load_coef(const StencilGeom& g, fx::W64 (*cf)[kStencilThreads]) {
-    fx::u64 b[5 * R];
-    int h = 0;
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-#pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        b[5 * r + k] = row_in(r) ? fx::d_bits(g.kc[k * g.J + q0 + r * m]) : 0;
-        h = max(h, fx::d_habs(b[5 * r + k]));
-      }
-    const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)h) >> 20;
-    const int Fc = max(e - 1022 - 62, fx::kFxMin);        // |coefficient| < 2^(e - 1022)
-    cs = e == 0x7FF ? kNoScale : Fc + 64;
-#pragma unroll
-    for (int i = 0; i < 5 * R; ++i) {
-      fx::i64 w = fx::d_to_fx(b[i], Fc);
-      if ((int)w == (int)0x80000000) ++w;                 // the low word can be negated
-      cf[i][threadIdx.x] = fx::split64(w);
-    }
-  }
-  // y = rows of v + tau K v - v^{n-1}.  |v| < 2^59 and |coefficient| < 2^62: the
-  // five products sum to less than 2^60
-  __device__ __forceinline__ void step_var(const Raw& w, const double* __restrict__ vs, const StencilGeom& g,
-                                           const fx::W64 (*cf)[kStencilThreads], int n, double (&y)[R]) {
-    using fx::i64;
-    const int e = q1_max(w), em = max(e, ep);
-    const int F = max(em - 1081, fx::kFxMin), s = cs, G = F + max(s, 0);
-    if (F != Fp) {
-#pragma unroll
-      for (int r = 0; r < R; ++r) prev[r] = fx::shift(prev[r], F - Fp);
-    }
-    const i64 rnd = s == 0 ? 0 : 1LL << (min(abs(s), 60) - 1);
-    const bool plain = em != 0x7FF && s != kNoScale && fx::fx_normal(G);
-    const i64 edge = fx::d_to_fx(w.edge, F);
-    i64 below = fx::d_to_fx(w.b[0], F), c = fx::d_to_fx(w.b[1], F);
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const i64 above = fx::d_to_fx(w.b[r + 2], F);
-      i64 le = __shfl_up_sync(0xffffffffu, c, 1), ri = __shfl_down_sync(0xffffffffu, c, 1);
-      const i64 ed = __shfl_sync(0xffffffffu, edge, lane < 16 ? r : R + r);
-      if (lane == 0) le = ed;
-      if (lane == 31) ri = ed;
-      const fx::W64* k = &cf[5 * r][threadIdx.x];
-      const i64 t = (fx::mul64(c, k[0]) - (fx::mul64(le, k[kStencilThreads]) + fx::mul64(ri, k[2 * kStencilThreads]))) -
-                    (fx::mul64(below, k[3 * kStencilThreads]) + fx::mul64(above, k[4 * kStencilThreads]));
-      const i64 d = c - prev[r];
-      prev[r] = c;
-      if (plain) y[r] = fx::fx_to_d(s >= 0 ? t + fx::shr(d + rnd, s) : fx::shr(t + rnd, -s) + d, G);
-      below = c;
-      c = above;
-    }
-    if (!plain) {
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-        y[r] = row_in(r) ? fx_slow_row<KIND, P>(vs, q0 + r * m, x, y0 + r, z0, n, g) : 0.0;
-    }
-    ep = e;
-    Fp = F;
-  }
   // y = row values of the slice vs = v^n, whose values are in w
   __device__ __forceinline__ void step(const Raw& w, const double* __restrict__ vs, const StencilGeom& g,
                                        const FxStencil& f, int n, double (&y)[R]) {
@@ -763,7 +689,6 @@ stencil_fx_kernel(const double* __restrict__ z, const double* __restrict__ aux, 
   double acc[NA];
 #pragma unroll
   for (int v = 0; v < NA; ++v) acc[v] = 0.0;
-  __shared__ fx::W64 cf[Row::VAR ? 5 * R : 1][kStencilThreads];
   const int lane = threadIdx.x & 31;
   const double ss = sshift ? sshift[0] : (MODE == kModeApply ? 1.0 : 0.0);
   const int wstep = gridDim.x * (kStencilThreads / 32), per = f.xt * f.yg * f.planes;
@@ -771,7 +696,6 @@ stencil_fx_kernel(const double* __restrict__ z, const double* __restrict__ aux, 
   for (int t = blockIdx.x * (kStencilThreads / 32) + (threadIdx.x >> 5); t < f.tiles; t += wstep) {
     const int tc = t / per;
     row.start(g, f, t - tc * per, lane);
-    if constexpr (Row::VAR) row.load_coef(g, cf);
     const int n0 = tc * f.chunk, n1 = min(g.N, n0 + f.chunk);
     const double* zs = z + (long long)n0 * g.J;
     typename Row::Raw cur, nxt;
@@ -795,7 +719,6 @@ stencil_fx_kernel(const double* __restrict__ z, const double* __restrict__ aux, 
       }
       double y[R];
       if constexpr (Row::Q1) row.step_q1(cur, zs, g, f, n, y);
-      else if constexpr (Row::VAR) row.step_var(cur, zs, g, cf, n, y);
       else row.step(cur, zs, g, f, n, y);
 #pragma unroll
       for (int r = 0; r < R; ++r) {
@@ -921,12 +844,12 @@ void stencil_dots_launch(int var, cudaStream_t st, const double* z, double* w,
 #undef BEC_SD_LAUNCH
 }
 
-// The fixed-point rows take 2D and 3D problems from 31 points a side (a warp's 32
-// columns are then nearly full); with the two-step scheme, finite differences
-// with a constant coefficient only.
+// The fixed-point rows take constant coefficients in 2D and 3D from 31 points a
+// side (a warp's 32 columns are then nearly full): finite differences, and Q1
+// elements (2D) with the one-step scheme.
 bool fx_rows(const bec_problem* p) {
-  return p->dim >= 2 && p->m >= 31 &&
-         (p->desc.time_scheme != BEC_TIME_BDF2 || (p->desc.space == BEC_SPACE_FD && p->kcoef == nullptr));
+  return p->kcoef == nullptr && p->dim >= 2 && p->m >= 31 &&
+         (p->desc.space == BEC_SPACE_FD || p->desc.time_scheme != BEC_TIME_BDF2);
 }
 
 // w = v 2^(63 - ce), |v| < 2^ce, as two words
@@ -973,7 +896,6 @@ void stencil_fx_launch(const bec_problem* p, unsigned grid, const double* z, con
       z, aux, w, g, f, L, vshift, sshift, p->partials)
   if (p->dim == 3) BEC_SFX(kFD3, 1);
   else if (p->desc.space == BEC_SPACE_Q1) BEC_SFX(kQ1, 1);
-  else if (p->kcoef != nullptr) BEC_SFX(kFDV, 1);
   else if (p->desc.time_scheme == BEC_TIME_BDF2) BEC_SFX(kFD, 2);
   else BEC_SFX(kFD, 1);
 #undef BEC_SFX
