@@ -427,8 +427,8 @@ __global__ void build_rhs_kernel(const double* __restrict__ u0, const double* __
 }
 
 // ---------------------------------------------------------------- fixed point
-// The finite-difference rows of L in 64-bit fixed point (bec_fx.cuh), 2D and
-// 3D with a constant coefficient.
+// The rows of L in 64-bit fixed point (bec_fx.cuh) with a constant coefficient:
+// finite differences in 2D and 3D, Q1 elements in 2D.
 //
 // GB300 issues 2 FP64 operations a clock and SM: the 5 (2D) or 7 (3D) of a row
 // bound the kernels above, whose vectors' traffic takes a quarter of that time.
@@ -446,6 +446,15 @@ __global__ void build_rhs_kernel(const double* __restrict__ u0, const double* __
 // Measured at 255^2 x 256: w = L z - s v with 1 and 2 dots 161 us on average
 // (FP64 rows: 287), ||f - L u|| 116 us (300); what bounds them now is the FP64
 // pipe again (2 operations and one a dot), 70 to 80 % busy.
+//
+// Q1 rows take six products, three of them by M, which the next step's row
+// subtracts: a lane keeps M v^{n-1} instead of the values.  At 127^2 x 64 (1M
+// unknowns) L v takes 20 us (FP64 rows: 56), ||f - L u|| 24 us (61).
+//
+// Variable coefficients keep the FP64 rows: five products on the tile's own
+// scale took w and its dots from 390 to 340 us at 255^2 x 256 (3 % of a
+// multigrid solve), and the other rounding of L moved solutions of the FP32
+// multigrid solves by up to 2e-10.
 constexpr int kFxRows = 4;
 constexpr int kFxDotVecs = 8;        // vectors a fused launch takes; more go to dots_kernel
 
