@@ -242,9 +242,7 @@ bec_status bec_allocate_problem(const bec_problem_desc* d, void* stream, bec_pro
   t.time.n = N;
   t.time.logn = ilog2(N);
   const long long U = p->U;
-  const long long parts = std::max<long long>(
-      std::max<long long>((long long)kMaxVec * kReduceBlocks, (long long)kMaxVec * kStencilDotBlocks),
-      2 * stencil_blocks(p));
+  const long long parts = partials_size(stencil_blocks(p));
   bec_status s = BEC_OK;
   auto chain = [&](bec_status r) {
     if (s == BEC_OK) s = r;

@@ -473,6 +473,14 @@ bec_status launch_stencil_dots(bec_problem* p, const double* z, double* w,
                                const double* sshift = nullptr, int norm_slot = -1);
 bec_status launch_build_rhs(bec_problem* p, const double* u0,
                             const double* fsrc, double* f);
+// Length of bec_problem::partials for the largest of its writers: the fused
+// stencil + dots pass, kStencilDotBlocks block sums of up to kMaxVec dots and of
+// ||w||^2, and the pairs of launch_residual_norms, one a block.
+inline long long partials_size(long long blocks) {
+  const long long dots = (long long)(kMaxVec + 1) * kStencilDotBlocks;
+  static_assert(kReduceBlocks <= kStencilDotBlocks, "the Krylov passes' sums fit with them");
+  return dots > 2 * blocks ? dots : 2 * blocks;
+}
 // partials[b] = sum over block b of (f - L u)^2, partials[B + b] = sum f^2;
 // then scal[slot] = sqrt(sum r^2), scal[slot+1] = sqrt(sum f^2).
 // fslot >= 0: ||f|| is in scal[fslot] and is copied instead; to_host: as launch_norm.
