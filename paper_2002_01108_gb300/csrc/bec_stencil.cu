@@ -439,9 +439,11 @@ __global__ void build_rhs_kernel(const double* __restrict__ u0, const double* __
 // A warp owns 32 columns and kFxRows rows of one slice (3D: of one plane) and
 // walks a chunk of time steps.  A lane converts its rows and the two beside
 // them once and gets its x neighbours by shuffle; only the edge lanes load one
-// more value a row.  The unit is a power of two from the largest value the
-// warp has loaded for the step and the one before, so that |v| < 2^59: the
-// error is below 2^-55 c max|v| of the tile, less than an FP64 row's.  Values
+// more value a row.  The unit is a power of two from the largest value of the
+// tile in the steps that the row takes (v^n, v^{n-1}; two-step scheme: v^{n-2}),
+// so that |v| < 2^59: the error is below 2^-55 c times that value.  The steps
+// before v^n are carried as bit patterns and converted in each row's own unit: an
+// integer in the unit of the row before would have lost bits to v^{n-2}.  Values
 // that are not finite or leave the range go through the FP64 row.
 // Measured at 255^2 x 256: w = L z - s v with 1 and 2 dots 161 us on average
 // (FP64 rows: 287), ||f - L u|| 116 us (300); what bounds them now is the FP64
@@ -492,8 +494,10 @@ struct FxRow {
   int m, lane, x, y0, z0, rows;
   unsigned in;               // which of b[] lie inside the domain; bit 31: the edge value
   long long q0, eo;          // the lane's first row; its edge value's point
+  // v^{n-1} (and v^{n-2}) of the rows as bit patterns: every row takes them in its
+  // own unit.  Q1: M v^{n-1} in the unit 2^Fp of v^{n-1} alone.
   fx::i64 prev[R], prev2[P == 2 ? R : 1];
-  int Fp, Fp2, ep, ep2;      // unit and largest exponent field of prev, prev2
+  int Fp, ep, ep2;           // Q1: unit of prev; largest exponent fields of v^{n-1}, v^{n-2}
 
   __device__ __forceinline__ void start(const StencilGeom& g, const FxStencil& f, int t, int ln) {
     lane = ln;
@@ -531,18 +535,15 @@ struct FxRow {
     }
   }
   // the centre values of a slice (zeros where there is none)
-  __device__ __forceinline__ void load_prev(const double* __restrict__ vs, fx::i64 (&pv)[R], int& F, int& e) {
-    fx::u64 b[R];
+  __device__ __forceinline__ void load_prev(const double* __restrict__ vs, fx::i64 (&pv)[R], int& e) {
     int h = 0;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      b[r] = vs != nullptr && row_in(r) ? fx::d_bits(vs[q0 + r * m]) : 0;
-      h = max(h, fx::d_habs(b[r]));
+      const fx::u64 b = vs != nullptr && row_in(r) ? fx::d_bits(vs[q0 + r * m]) : 0;
+      pv[r] = (fx::i64)b;
+      h = max(h, fx::d_habs(b));
     }
     e = (int)__reduce_max_sync(0xffffffffu, (unsigned)h) >> 20;
-    F = max(e - 1081, fx::kFxMin);
-#pragma unroll
-    for (int r = 0; r < R; ++r) pv[r] = fx::d_to_fx(b[r], F);
   }
   // Q1: visit(r, centre, sum of the 4 edge neighbours, of the 4 corners) for the
   // rows of a slice, in the unit 2^F
@@ -587,19 +588,18 @@ struct FxRow {
     Fp = max(ep - 1081, fx::kFxMin);
     q1_rows(w, Fp, [&](int r, fx::i64 c, fx::i64 e, fx::i64 d) { prev[r] = q1_form(f.wm, c, e, d); });
   }
-  // y = rows of (M + tau K) v^n - M v^{n-1}.  |v| < 2^59 and |coefficient| < 2^63:
-  // each of the two parts stays below 2^61.2
+  // y = rows of (M + tau K) v^n - M v^{n-1}.  Each part is formed in the unit of
+  // its own slice (|v| < 2^59 and |coefficient| < 2^63: below 2^61.2); the finer
+  // one is rounded to the other's unit, so that a row sees its own operands only.
   __device__ __forceinline__ void step_q1(const Raw& w, const double* __restrict__ vs, const StencilGeom& g,
                                           const FxStencil& f, int n, double (&y)[R]) {
     const int e = q1_max(w), em = max(e, ep);
-    const int F = max(em - 1081, fx::kFxMin), G = F + f.ce + 1;
-    if (F != Fp) {
-#pragma unroll
-      for (int r = 0; r < R; ++r) prev[r] = fx::shift(prev[r], F - Fp);
-    }
+    const int F = max(e - 1081, fx::kFxMin), G = max(F, Fp) + f.ce + 1;
+    const int da = min(max(Fp - F, 0), 63), dp = min(max(F - Fp, 0), 63);
+    const fx::i64 ra = da > 0 ? 1LL << (da - 1) : 0, rp = dp > 0 ? 1LL << (dp - 1) : 0;
     const bool plain = em != 0x7FF && fx::fx_normal(G);
     q1_rows(w, F, [&](int r, fx::i64 c, fx::i64 eg, fx::i64 d) {
-      const fx::i64 Y = q1_form(f.wa, c, eg, d) - prev[r];
+      const fx::i64 Y = fx::shr(q1_form(f.wa, c, eg, d) + ra, da) - fx::shr(prev[r] + rp, dp);
       prev[r] = q1_form(f.wm, c, eg, d);
       if (plain) y[r] = fx::fx_to_d(Y, G);
     });
@@ -627,24 +627,16 @@ struct FxRow {
     const int F = max(em - 1081, fx::kFxMin);            // |v| < 2^(em - 1022) = 2^(F + 59)
     const int s = f.ce + 1;                               // c lap = mul64(lap, cm) 2^s
     const int G = F + max(s, 0);
+    if constexpr (P == 2) ep2 = ep;
+    ep = e;
     if (em == 0x7FF || !fx::fx_normal(G)) {
 #pragma unroll
-      for (int r = 0; r < R; ++r)
+      for (int r = 0; r < R; ++r) {
         y[r] = row_in(r) ? fx_slow_row<KIND, P>(vs, q0 + r * m, x, y0 + r, z0, n, g) : 0.0;
-      ep = e;
-      Fp = F;
-#pragma unroll
-      for (int r = 0; r < R; ++r) prev[r] = fx::d_to_fx(w.b[r + 1], F);
-      if constexpr (P == 2) load_prev(n > 0 ? vs - g.J : nullptr, prev2, Fp2, ep2);
+        if constexpr (P == 2) prev2[r] = prev[r];
+        prev[r] = (i64)w.b[r + 1];
+      }
       return;
-    }
-    if (F != Fp) {
-#pragma unroll
-      for (int r = 0; r < R; ++r) prev[r] = fx::shift(prev[r], F - Fp);
-    }
-    if (P == 2 && F != Fp2) {
-#pragma unroll
-      for (int r = 0; r < (P == 2 ? R : 0); ++r) prev2[r] = fx::shift(prev2[r], F - Fp2);
     }
     // shifts round to nearest: a bias of even a small part of a unit, the same at
     // every point, would come back from L^{-1} many times larger
@@ -663,24 +655,18 @@ struct FxRow {
       const i64 t = fx::mul64(lap, f.cm);
       i64 Y;
       if constexpr (P == 2) {                             // (3 v - 4 v' + v'') / 2
-        const i64 d = 3 * c - 4 * prev[r] + prev2[r];
+        const i64 d = 3 * c - 4 * fx::d_to_fx((fx::u64)prev[r], F) + fx::d_to_fx((fx::u64)prev2[r], F);
         Y = s >= 0 ? t + fx::shr(d + (1LL << s), s + 1) : fx::shr(t + rnd, -s) + ((d + 1) >> 1);
         prev2[r] = prev[r];
       } else {
-        const i64 d = c - prev[r];
+        const i64 d = c - fx::d_to_fx((fx::u64)prev[r], F);
         Y = s >= 0 ? t + fx::shr(d + rnd, s) : fx::shr(t + rnd, -s) + d;
       }
-      prev[r] = c;
+      prev[r] = (i64)w.b[r + 1];
       y[r] = fx::fx_to_d(Y, G);
       below = c;
       c = above;
     }
-    if constexpr (P == 2) {
-      ep2 = ep;
-      Fp2 = F;
-    }
-    ep = e;
-    Fp = F;
   }
 };
 
@@ -710,9 +696,9 @@ stencil_fx_kernel(const double* __restrict__ z, const double* __restrict__ aux, 
     typename Row::Raw cur, nxt;
     row.load(zs, cur);
     if constexpr (Row::Q1) row.load_prev_q1(n0 > 0 ? zs - g.J : nullptr, f);
-    else row.load_prev(n0 > 0 ? zs - g.J : nullptr, row.prev, row.Fp, row.ep);
+    else row.load_prev(n0 > 0 ? zs - g.J : nullptr, row.prev, row.ep);
     if constexpr (P == 2)
-      row.load_prev(n0 > 1 ? zs - 2 * g.J : nullptr, row.prev2, row.Fp2, row.ep2);
+      row.load_prev(n0 > 1 ? zs - 2 * g.J : nullptr, row.prev2, row.ep2);
     long long o0 = (long long)n0 * g.J + row.q0;
     for (int n = n0; n < n1; ++n) {
       // the next slice's values and this one's other operands are on their way
