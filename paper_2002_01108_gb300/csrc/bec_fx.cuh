@@ -364,6 +364,8 @@ BEC_FX unsigned f_bits(float f) {
   return u;
 #endif
 }
+// 2^e for e < 128, at least 2^-126
+BEC_FX float exp2_f(int e) { return bits_f((unsigned)(e < -126 ? 1 : e + 127) << 23); }
 BEC_FX int ilog2f(float f) { return (int)(f_bits(f) >> 23) - 127; }                       // f > 0
 
 // v >> 32 >> d as a float's magnitude, in units 2^(32 + the reference exponent)
@@ -499,16 +501,29 @@ BEC_FX i64 shr(i64 v, int r) {
   return v >> (r > 63 ? 63 : r);
 #endif
 }
+// v 2^r, 0 from r = 64 on
+BEC_FX i64 shl(i64 v, int r) {
+#ifdef __CUDA_ARCH__
+  i64 d;
+  asm("shl.b64 %0, %1, %2;" : "=l"(d) : "l"(v), "r"(r));
+  return d;
+#else
+  return r > 63 ? 0 : (i64)((u64)v << r);
+#endif
+}
 // v 2^-r for either sign of r
 BEC_FX i64 shift(i64 v, int r) {
   const int l = r < 0 ? -r : 0, k = r < 0 ? 0 : r;
-#ifdef __CUDA_ARCH__
-  i64 d;
-  asm("shl.b64 %0, %1, %2;" : "=l"(d) : "l"(v), "r"(l));
-  return shr(d, k);
-#else
-  return shr((i64)((u64)v << (l > 63 ? 63 : l)), k);
-#endif
+  return shr(shl(v, l), k);
+}
+// the same rounded to nearest, |v| < 2^62 (0 from r = 63 on)
+BEC_FX i64 shr_rn(i64 v, int r) {
+  const int k = r < 63 ? r : 63;
+  return shr(v + (i64)((u64)shl(1, k) >> 1), k);
+}
+BEC_FX i64 shift_rn(i64 v, int r) {
+  const int l = r < 0 ? -r : 0, k = r < 0 ? 0 : r;
+  return shr_rn(shl(v, l), k);
 }
 BEC_FX u64 shr_u(u64 v, int r) {
 #ifdef __CUDA_ARCH__

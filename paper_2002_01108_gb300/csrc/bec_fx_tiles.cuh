@@ -453,7 +453,7 @@ struct TimeArgs {
   const double* eis;           // eps^{-j/N}
   const double* scale_dev;     // null: 1
   const CW64* q;               // [N/2+1][J]: scale conj(d) / |d|^2, times 2^(63 - qe)
-  const int* qe;               // one a tile
+  const int* qe;               // [tile][N/2+1]
   const CW64* tw;
 };
 
@@ -488,7 +488,8 @@ struct TimeTile {
   static constexpr size_t kBuf = (size_t)LPB * G::STRIDE * sizeof(cx);
   static constexpr size_t kStat = (size_t)THREADS * sizeof(Stat);
   static constexpr size_t kMax = (size_t)THREADS * sizeof(int);
-  static constexpr size_t SMEM = kBuf + kStat + kMax + (size_t)N * (sizeof(W64) + sizeof(int)) + LPB * sizeof(int);
+  static constexpr size_t SMEM = kBuf + kStat + kMax + (size_t)N * (sizeof(W64) + sizeof(int)) +
+                                 (LPB + N / 2 + 1) * sizeof(int);
   using Join = LineJoin<LPB, TPL, false>;
   static constexpr int R1 = 1 << radix_log(LOGN, 0);
   static constexpr int RL = 1 << radix_log(LOGN, G::NP - 1);
@@ -498,6 +499,7 @@ struct TimeTile {
     Stat* st;
     int *mx, *fl, *se;                              // se[j]: exponent of time step j's values
     W64* eim;                                       // eps^{-j/N} scale, as mantissas
+    int* qx;                                        // qe[k] - qe[0]; null: no factors
     int L, t, tid;
     bool va, vb;
     long long qa, qb, tile;
@@ -521,6 +523,7 @@ struct TimeTile {
     c.eim = reinterpret_cast<W64*>(smem + kBuf + kStat + kMax);
     c.se = reinterpret_cast<int*>(c.eim + N);
     c.fl = c.se + N;
+    c.qx = nullptr;
     const int XG = (m + W) / W;                     // m + 1 = a power of two >= W, or 1
     const long long row = blk / XG;
     const int xg = (int)(blk - row * XG), x0 = xg * W + c.L;
@@ -548,6 +551,12 @@ struct TimeTile {
     max_put<THREADS>(c.mx, tid, e);
   }
 
+  // the exponents of the factors; after load(), whose loads are then on their way
+  static BEC_FX void factors(Ctx& c, const TimeArgs& g) {
+    c.qx = c.fl + LPB;
+    const int* qe = g.qe + c.tile * (N / 2 + 1);
+    for (int k = c.tid; k < N / 2 + 1; k += THREADS) c.qx[k] = qe[k] - qe[0];
+  }
   template <typename Args>
   static BEC_FX void load(Ctx& c, Reg& r, const Args& g) {
     int b0, step;
@@ -665,12 +674,19 @@ struct TimeTile {
       cx nc;
       divide(C, C, qa[N / 2 * g.J], qb[N / 2 * g.J], nc, r.v[1]);
     }
+    // the products at k count in the unit 2^qe[k], the statistics in 2^qe[0]
     float m = 0.f, l = 0.f;
 #pragma unroll
-    for (int i = 0; i < EPT; ++i) {
-      const float x = mag(r.v[i].x), y = mag(r.v[i].y);
-      m = fmaxf(m, fmaxf(x, y));
-      l += x + y;
+    for (int u = 0; u < H; ++u) {
+      const float w = exp2_f(c.qx[c.t + TPL * u]);
+      const float w1 = u == 0 && c.t == 0 ? exp2_f(c.qx[N / 2]) : w;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const float x = mag(r.v[2 * u + i].x), y = mag(r.v[2 * u + i].y);
+        // one unit of slack each
+        m = fmaxf(m, (fmaxf(x, y) + 1.f) * (i == 0 ? w : w1));
+        l += (x + y + 2.f) * (i == 0 ? w : w1);
+      }
     }
     c.s = {m, l};
     Join::put(c.st, c.s, c.tid, c.L);
@@ -678,21 +694,20 @@ struct TimeTile {
   // the solution spectrum on the inverse transform's scale, parts exchanged
   static BEC_FX void rescale(Ctx& c, Reg& r) {
     const Stat s = Join::get(c.st, c.s, c.tid, c.L);
-    const Scale k = line_scale<LOGN>(0, (float)R1 * 1.4143f * (s.m + 1.f), s.l + (float)(2 * N));
+    const Scale k = line_scale<LOGN>(0, (float)R1 * 1.4143f * s.m, s.l);
     c.sc = k;
     c.f += 1 + k.F + k.s2 + k.s3;                   // 1: q halves
     if (c.t == 0) c.fl[c.L] = c.f;
-    const int kl = k.F < 0 ? -k.F : 0, kr = k.F < 0 ? 0 : k.F;
-    const i64 rnd = kr > 0 ? 1LL << (kr - 1) : 0;
     cx* fp = c.line + slot(c.t);
 #pragma unroll
     for (int u = 0; u < H; ++u) {
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
-        const cx v = r.v[2 * u + i];
-        const cx w{shr((v.y << kl) + rnd, kr), shr((v.x << kl) + rnd, kr)};
+        const bool mid = i == 1 && u == 0 && c.t == 0;
+        const int d = c.qx ? k.F - c.qx[mid ? N / 2 : c.t + TPL * u] : k.F;
+        const cx v = r.v[2 * u + i], w{shift_rn(v.y, d), shift_rn(v.x, d)};
         if (i == 0) fp[slot(TPL * u)] = w;
-        else c.line[slot(u == 0 && c.t == 0 ? N / 2 : N - c.t - TPL * u)] = w;
+        else c.line[slot(mid ? N / 2 : N - c.t - TPL * u)] = w;
       }
     }
   }
@@ -718,7 +733,7 @@ struct TimeTile {
       if (c.va) pa[j * g.J] = mul64(shr(r.v[i].y + rnd, d), w);
       if (c.vb) pb[j * g.J] = mul64(shr(r.v[i].x + rnd, d), w);
     }
-    if (c.tid == 0) g.eout[c.tile] = fm + 1 + g.qe[c.tile];
+    if (c.tid == 0) g.eout[c.tile] = fm + 1 + g.qe[c.tile * (N / 2 + 1)];
   }
 };
 
@@ -871,8 +886,8 @@ struct SpecTile : TimeTile<LOGN, LPB> {
 #pragma unroll
     for (int i = 0; i < EPT; ++i) {
       const float x = mag(r.v[i].x), y = mag(r.v[i].y);
-      m = fmaxf(m, fmaxf(x, y));
-      l += x + y;
+      m = fmaxf(m, fmaxf(x, y) + 1.f);              // one unit of slack each
+      l += x + y + 2.f;
     }
     c.s = {m, l};
     Join::put(c.st, c.s, c.tid, c.L);

@@ -32,6 +32,7 @@ __global__ void __launch_bounds__(Tile::THREADS, fxt_blocks(Tile::THREADS)) time
   typename Tile::Reg r;
   Tile::init(c, g, fx_smem, tid, blockIdx.x);
   Tile::load(c, r, g);
+  Tile::factors(c, g);
   __syncthreads();
   Tile::measure(c, r);
   __syncthreads();
@@ -145,8 +146,10 @@ bec_status fx_spec(bec_problem* p, const SpecArgs& g) {
 }
 
 // q[k][q] = scale conj(d) / |d|^2 with d = lambda'_k mu^M + tau mu^K, times
-// 2^(63 - qe): the smallest |d| of the W modes of a tile (W lanes) sets qe so
-// that |q| stays below 0.9.
+// 2^(63 - qe[k]): the largest |q| of the W modes of a tile (W lanes) at k sets
+// qe[tile][k] so that |q| stays below 0.9.  With one exponent for all k, that of
+// the smallest |d|, the factors of the high frequencies would keep only 63 -
+// log2(|d_k| / |d_0|) bits: 41 at eps = 1 and a = 1e-5.
 template <int W>
 __global__ void fx_table_kernel(CW64* __restrict__ q, int* __restrict__ qe, long long rows, int xg,
                                 long long J, int NK, int m, int dim, const double2* __restrict__ lamf,
@@ -159,25 +162,23 @@ __global__ void fx_table_kernel(CW64* __restrict__ q, int* __restrict__ qe, long
   double muM, muK;
   mode_eigs(i, J, m, m, dim, me, muM, muK);
   const bool fe = me.m != nullptr;
-  // Re lambda'_k grows with k on [0, N/2] for both schemes and is >= 0 at k = 0,
-  // where Im lambda'_k = 0: the smallest |d| is d_0
-  const double d0 = fe ? fma(lamf[0].x, muM, tau * muK) : lamf[0].x + tau * muK;
-  int e;
-  if (frexp(scale / d0, &e) > 0.9) ++e;
-  if (!in) e = -kFxNan;
-#pragma unroll
-  for (int o = 1; o < W; o <<= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-  if (!in) return;
-  if (x % W == 0) qe[row * xg + x / W] = e;
-  auto fixed = [e](double v) {
-    i64 w = d_to_fx(d_bits(v), e - 63);
-    if ((int)w == (int)0x80000000) ++w;          // the low word can be negated
-    return split64(w);
-  };
+  int* tile_qe = qe + (row * xg + x / W) * NK;
   for (int k = 0; k < NK; ++k) {
     const double2 L = lamf[k];
     const double dr = fe ? fma(L.x, muM, tau * muK) : L.x + tau * muK, di = fe ? L.y * muM : L.y;
     const double s = scale / fma(dr, dr, di * di);
+    // |q|^2 = scale s < 2^(E - 1022) with E its exponent field; / 0.81 in [1, 2)
+    int e = (((int)(fx::d_bits(scale * s * (1.0 / 0.81)) >> 52) - 1022 + 1) >> 1);
+    if (!in) e = -kFxNan;
+#pragma unroll
+    for (int o = 1; o < W; o <<= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+    if (!in) continue;
+    if (x % W == 0) tile_qe[k] = e;
+    auto fixed = [e](double v) {
+      i64 w = d_to_fx(d_bits(v), e - 63);
+      if ((int)w == (int)0x80000000) ++w;        // the low word can be negated
+      return split64(w);
+    };
     q[(long long)k * J + i] = CW64{fixed(dr * s), fixed(di * s)};
   }
 }
@@ -260,7 +261,7 @@ bec_status fx_setup(bec_problem* p) {
   const size_t o_ts = place(ts.size() * sizeof(CW64)), o_tt = place(tt.size() * sizeof(CW64));
   const size_t o_sin = place(sinw.size() * sizeof(W64)), fixed = size;
   const size_t o_esm = place(N * sizeof(W64)), o_ese = place(N * sizeof(int));
-  const size_t o_x = place(N * sizeof(int)), o_qe = place(tiles * sizeof(int));
+  const size_t o_x = place(N * sizeof(int)), o_qe = place(tiles * (N / 2 + 1) * sizeof(int));
   const size_t o_em = place(tiles * sizeof(int)), o_e0 = place(ne * sizeof(int)), o_e1 = place(ne * sizeof(int));
   cudaError_t e = cudaMalloc(&t.tables, size);
   if (e == cudaSuccess) e = cudaMalloc(&t.q, (size_t)p->J * (N / 2 + 1) * sizeof(CW64));

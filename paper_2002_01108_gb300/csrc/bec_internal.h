@@ -67,9 +67,9 @@ struct FxTables {
   void* tw_space = nullptr;  // scaled twiddles of n = nx + 1 and of N
   void* tw_time = nullptr;
   void* sinw = nullptr;      // 2 sin(j pi / n) - 1
-  void* q = nullptr;         // [N/2+1][J] complex: scale / (lambda'_k + tau mu_q), per mode 2^-qe
+  void* q = nullptr;         // [N/2+1][J] complex: scale / (lambda'_k + tau mu_q) times 2^(63 - qe)
   int lpb = 0;               // line pairs a block transforms
-  int* qe = nullptr;         // exponents of q, one a tile of 2 lpb modes
+  int* qe = nullptr;         // exponents of q: [tile of 2 lpb modes][N/2+1]
   int* e0 = nullptr;         // exponents of the tiles between the passes
   int* e1 = nullptr;
   int* em = nullptr;         // exponents of the time pass's tiles
