@@ -73,14 +73,14 @@ BEC_FX i64 mul64(i64 x, W64 w, i64 init = kHalf) {
 // x c + y d and y c - x d, divided by 2^64 (rounded): the product of x + i y
 // and c - i d.  The 64-bit sum of the four cross products stays below 2^63 for
 // |x + i y| < 2^62 and |c + i d| <= 0.9 2^63.
-BEC_FX cx cmul_conj(cx v, CW64 w) {
+BEC_FX cx cmul_conj(cx v, CW64 w, i64 ix = kHalf, i64 iy = kHalf) {
   const int xh = hi_r(v.x), xl = (int)v.x, yh = hi_r(v.y), yl = (int)v.y;
   const int nh = -w.d.h, nl = -w.d.l;
-  i64 m = madw(xh, w.c.l, kHalf);
+  i64 m = madw(xh, w.c.l, ix);
   m = madw(xl, w.c.h, m);
   m = madw(yh, w.d.l, m);
   m = madw(yl, w.d.h, m);
-  i64 n = madw(yh, w.c.l, kHalf);
+  i64 n = madw(yh, w.c.l, iy);
   n = madw(yl, w.c.h, n);
   n = madw(xh, nl, n);
   n = madw(xl, nh, n);
@@ -91,12 +91,12 @@ BEC_FX cx cmul_conj(cx v, CW64 w) {
 }
 // SIGN -1: v (c - i d); +1: v (c + i d), over 2^64
 template <int SIGN>
-BEC_FX cx cmul_w(cx v, CW64 w) {
+BEC_FX cx cmul_w(cx v, CW64 w, i64 ix, i64 iy) {
   if constexpr (SIGN > 0) {
     w.d.h = -w.d.h;              // no word of a table entry is -2^31
     w.d.l = -w.d.l;
   }
-  return cmul_conj(v, w);
+  return cmul_conj(v, w, ix, iy);
 }
 
 BEC_FX cx add(cx a, cx b) { return {a.x + b.x, a.y + b.y}; }
@@ -273,9 +273,14 @@ constexpr int tw_count(int logn) {
 constexpr int tw_first(int logn, int p) { return p == 0 ? 0 : kFxShifts << logn; }
 
 // The DFTs and twiddles of pass P on the thread's values: butterfly u of
-// thread t is b = t + TPL u, its element i at v[u R + i]; s: the pass's shift.
-template <int LOGN, int P, int SIGN>
-BEC_FX void pass_compute(cx (&v)[Line<LOGN>::EPT], const CW64* __restrict__ tw, int t, int s) {
+// thread t is b = t + TPL u, its element i at v[u R + i]; s: the pass's shift;
+// dx, dy: whether the real and the imaginary parts that are only shifted, and
+// with TIES the products (many are by powers of two), round ties down (0 or 1).
+// Ties that all go one way leave a mean, 1/8 of a unit an element at s = 2; lines
+// that a later transform adds up take turns, so that these means cancel.
+template <int LOGN, int P, int SIGN, bool TIES = false>
+BEC_FX void pass_compute(cx (&v)[Line<LOGN>::EPT], const CW64* __restrict__ tw, int t, int s,
+                         int dx = 0, int dy = 0) {
   using G = Line<LOGN>;
   constexpr int lr = radix_log(LOGN, P), R = 1 << lr, NB = G::EPT / R;
   constexpr int before = before_log(LOGN, P), lm = LOGN - before - lr;
@@ -289,9 +294,9 @@ BEC_FX void pass_compute(cx (&v)[Line<LOGN>::EPT], const CW64* __restrict__ tw, 
       const int i1 = (t + G::TPL * u) & ((1 << lm) - 1);
       const CW64* tp = tw + tw_first(LOGN, P) + ((s - 2) << (LOGN - before)) + i1;
       const i64 rnd = 1LL << (s - 1);
-      w[0] = {(w[0].x + rnd) >> s, (w[0].y + rnd) >> s};
+      w[0] = {(w[0].x + (rnd - dx)) >> s, (w[0].y + (rnd - dy)) >> s};
 #pragma unroll
-      for (int l = 1; l < R; ++l) w[l] = cmul_w<SIGN>(w[l], tp[l << lm]);
+      for (int l = 1; l < R; ++l) w[l] = cmul_w<SIGN>(w[l], tp[l << lm], TIES ? kHalf - dx : kHalf, TIES ? kHalf - dy : kHalf);
     }
 #pragma unroll
     for (int i = 0; i < R; ++i) v[u * R + i] = w[i];

@@ -75,6 +75,7 @@ struct DstTile {
     long long la, lb;                               // offsets of x_1 of the two lines
     long long es;                                   // elements from x_j to x_{j+1}
     int ref, add, f;                                // f: exponent of the line's outputs
+    int dx, dy;                                     // pass_compute; ROWS: constants
     Stat s;
     Scale sc;
   };
@@ -104,6 +105,8 @@ struct DstTile {
       c.la = ra * m;
       c.lb = c.la + m;
       c.es = 1;
+      c.dx = 0;                                     // rows in turn (m is odd: a row's steps too)
+      c.dy = 1;
       if constexpr (!IN_D) {
         for (int k = tid; k < NE; k += THREADS) {
           const long long r = r0 + k / XG;
@@ -125,6 +128,7 @@ struct DstTile {
       c.la = (z ? u / m * g.J + u % m * m : u * m * m) + ca;
       c.lb = c.la + LPB;
       c.es = z ? m * m : m;
+      c.dx = c.dy = (int)((z || g.dim == 3 ? u / m : u) & 1);   // time steps in turn
       if (g.kind == kColsYBack) c.add = g.xadd[g.dim == 2 ? u : u / m];
       for (int k = tid; k < n - 1; k += THREADS) {
         const int x = g.kind == kColsY ? g.ein[(u * m + k) / W]
@@ -279,32 +283,36 @@ struct DstTile {
 #pragma unroll
       for (int u = 0; u < H; ++u)
         if (k < 0)
-          pair(c, g, u, r.a[u] << -k, r.a2[u] << -k, r.b[u] << -k, r.b2[u] << -k, kHalf);
+          pair(c, g, u, r.a[u] << -k, r.a2[u] << -k, r.b[u] << -k, r.b2[u] << -k, 0);
         else
-          pair(c, g, u, r.a[u], r.a2[u], r.b[u], r.b2[u], kHalf);
+          pair(c, g, u, r.a[u], r.a2[u], r.b[u], r.b2[u], 0);
     } else {
-      // integers are shifted rounding down (mean -1/2 for x_j and x_{n-j}): h
-      // is rounded half a unit higher to make up for it
+      // integers are shifted rounding down by k (and more), which takes (1 - 2^-k) / 2
+      // of a unit from x_j and x_{n-j} in the mean and 1 + w_j times that from y_j: h
+      // gets it back.  A mean left in y would meet in the lowest modes, which the time
+      // pass amplifies.
       if (all_warp<THREADS>(k >= 0)) {              // right shifts only
 #pragma unroll
         for (int u = 0; u < H; ++u) {
           const Ex e = exps(c, u);
           pair(c, g, u, shr(r.a[u], fi - e.x), shr(r.a2[u], fi - e.x2), shr(r.b[u], fi - e.y),
-               shr(r.b2[u], fi - e.y2), k > 0 ? 2 * kHalf : kHalf);
+               shr(r.b2[u], fi - e.y2), k > 0 ? k : 0);
         }
       } else {
 #pragma unroll
         for (int u = 0; u < H; ++u) {
           const Ex e = exps(c, u);
           pair(c, g, u, shift(r.a[u], fi - e.x), shift(r.a2[u], fi - e.x2), shift(r.b[u], fi - e.y),
-               shift(r.b2[u], fi - e.y2), k > 0 ? 2 * kHalf : kHalf);
+               shift(r.b2[u], fi - e.y2), k > 0 ? k : 0);
         }
       }
     }
   }
   // y_p and y_{n-p}, p = t + TPL u, to shared memory
-  static BEC_FX void pair(const Ctx& c, const DstArgs& g, int u, i64 a, i64 a2, i64 b, i64 b2, i64 init) {
+  static BEC_FX void pair(const Ctx& c, const DstArgs& g, int u, i64 a, i64 a2, i64 b, i64 b2, int k) {
     const W64 w = g.sinw[c.t + TPL * u];
+    const unsigned back = 0x80000000u + (unsigned)w.h;    // (1 + w) / 2
+    const i64 init = kHalf + (i64)(back - (back >> (k < 31 ? k : 31)));
     const i64 sa = a + a2, sb = b + b2;
     const i64 ha = mul64(sa, w, init), hb = mul64(sb, w, init);   // s w / 2
     if (u == 0) {                                   // p = 0: y_{n/2} = 4 x_{n/2}, y_0 = 0
@@ -321,7 +329,7 @@ struct DstTile {
   template <int P>
   static BEC_FX void pass(Ctx& c, Reg& r, const DstArgs& g) {
     pass_read<LOGN, P>(r.v, c.line, c.t);
-    pass_compute<LOGN, P, -1>(r.v, g.tw, c.t, P == 0 ? c.sc.s2 : c.sc.s3);
+    pass_compute<LOGN, P, -1, ROWS>(r.v, g.tw, c.t, P == 0 ? c.sc.s2 : c.sc.s3, c.dx, c.dy);
     if constexpr (P + 1 < G::NP) pass_write<LOGN, P>(r.v, c.line, c.t);
   }
   static BEC_FX void natural(Ctx& c, Reg& r) { write_natural<LOGN>(r.v, c.line, c.t); }
@@ -369,15 +377,16 @@ struct DstTile {
     for (int i = 1; i < LPB; ++i) fm = fm > c.fl[i] ? fm : c.fl[i];
     const int d = fm - c.f;
     c.f = fm;
-    const i64 rnd = d > 0 ? 1LL << ((d > 62 ? 62 : d) - 1) : 0;
-    off = cx{off.x + rnd, off.y + rnd};
+    const i64 half = d > 0 ? 1LL << ((d > 62 ? 62 : d) - 1) : 0;
+    const cx rnd = d > 0 ? cx{half - c.dx, half - c.dy} : cx{0, 0};
+    off = add(off, rnd);
     auto dn = [d](i64 v) { return shr(v, d); };
     if constexpr (ROWS) {
       // line a, then line b, a pad slot every 16
       i64* ob = reinterpret_cast<i64*>(c.line) + (2 * H + 1) * c.t;
 #pragma unroll
       for (int i = 0; i < H; ++i) {
-        const cx od = add(r.v[2 * i], off), ev = add(r.v[2 * i + 1], cx{rnd, rnd});
+        const cx od = add(r.v[2 * i], off), ev = add(r.v[2 * i + 1], rnd);
         ob[2 * i] = dn(od.x);
         ob[RS + 2 * i] = dn(od.y);
         if (i > 0) {
@@ -394,14 +403,14 @@ struct DstTile {
 #pragma unroll
         for (int i = 0; i < H; ++i) {
           oa[2 * i * c.es] = dn(r.v[2 * i].x + off.x);
-          if (i > 0 || c.t > 0) oa[(2 * i - 1) * c.es] = dn(r.v[2 * i + 1].x + rnd);
+          if (i > 0 || c.t > 0) oa[(2 * i - 1) * c.es] = dn(r.v[2 * i + 1].x + rnd.x);
         }
       }
       if (c.vb) {
 #pragma unroll
         for (int i = 0; i < H; ++i) {
           ob[2 * i * c.es] = dn(r.v[2 * i].y + off.y);
-          if (i > 0 || c.t > 0) ob[(2 * i - 1) * c.es] = dn(r.v[2 * i + 1].y + rnd);
+          if (i > 0 || c.t > 0) ob[(2 * i - 1) * c.es] = dn(r.v[2 * i + 1].y + rnd.y);
         }
       }
     }
@@ -609,7 +618,8 @@ struct TimeTile {
     c.sc = line_scale<LOGN>(c.ref, (float)R1 * 1.4143f * (s.m + 1.f), 2.f * (s.l + (float)N));
     const int fi = c.sc.F - 1;                      // eps^{j/N} times 2^63: half
     const int k = fi - c.ref;
-    const i64 init = k > 0 ? kHalf + kHalf / 2 : kHalf;
+    // shifts round to nearest: a mean left here is frequency 0's, whose factor is
+    // the largest
     int b0, step;
     bfly_index<LOGN, 0>(c.t, b0, step);
     const W64* wp = g.esm + b0;
@@ -621,7 +631,7 @@ struct TimeTile {
         bfly_index<LOGN, 0>(TPL * (i / R1), bu, st);
         const int j = bu + (i % R1) * st, d = fi - ep[j];
         const W64 w = wp[j];
-        r.v[i] = cx{mul64(shr(r.v[i].x, d), w, init), mul64(shr(r.v[i].y, d), w, init)};
+        r.v[i] = cx{mul64(shr_rn(r.v[i].x, d), w), mul64(shr_rn(r.v[i].y, d), w)};
       }
     } else {
 #pragma unroll
@@ -630,7 +640,7 @@ struct TimeTile {
         bfly_index<LOGN, 0>(TPL * (i / R1), bu, st);
         const int j = bu + (i % R1) * st, d = fi - ep[j];
         const W64 w = wp[j];
-        r.v[i] = cx{mul64(shift(r.v[i].x, d), w, init), mul64(shift(r.v[i].y, d), w, init)};
+        r.v[i] = cx{mul64(shift_rn(r.v[i].x, d), w), mul64(shift_rn(r.v[i].y, d), w)};
       }
     }
     c.f = (c.ref > kFxNan / 2 ? kFxNan : c.sc.F) + c.sc.s2 + c.sc.s3;
@@ -833,8 +843,7 @@ struct SpecTile : TimeTile<LOGN, LPB> {
       int bu, st;
       bfly_index<LOGN, 0>(TPL * (i / R1), bu, st);
       const int j = b0 + bu + (i % R1) * st, d = fi - c.ref - c.se[j];
-      const i64 init = d > 0 ? kHalf + kHalf / 2 : kHalf;
-      r.v[i] = cx{mul64(shift(r.v[i].x, d), c.eim[j], init), mul64(shift(r.v[i].y, d), c.eim[j], init)};
+      r.v[i] = cx{mul64(shift_rn(r.v[i].x, d), c.eim[j]), mul64(shift_rn(r.v[i].y, d), c.eim[j])};
     }
     if (e > kFxNan / 2) c.f = kFxNan;
     c.f += (c.f == kFxNan ? 0 : c.sc.F) + c.sc.s2 + c.sc.s3;
