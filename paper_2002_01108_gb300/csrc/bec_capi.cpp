@@ -469,7 +469,7 @@ bec_status bec_apply_A(bec_problem* p, const double* v, double* y) {
   BEC_TRY(check_vec(v));
   BEC_TRY(check_vec(y));
   if (overlap(p, v, y)) return einval("v and y must not overlap");
-  return launch_apply_L(p, v, y, 0.0);
+  return launch_apply_L(p, v, y, 0.0, nullptr, true);
 }
 
 bec_status bec_apply_P(bec_problem* p, const double* v, double* y) {

@@ -461,8 +461,10 @@ bec_status net_judge_radii(bec_problem* p, double* host);
 long long stencil_blocks(const bec_problem* p);
 // y = L v; with corner != 0, y = P_eps v (adds -corner * v^N to slice 1);
 // with out_scale != null the result is multiplied by the device scalar.
+// own: every row is as accurate as in FP64 for its own values, not in norm alone
+// (FxRow).
 bec_status launch_apply_L(bec_problem* p, const double* v, double* y,
-                          double corner, const double* out_scale = nullptr);
+                          double corner, const double* out_scale = nullptr, bool own = false);
 // w = L z - s vshift (s = *sshift; no shift if vshift is null) and
 // hout[i] = sigma_i <V_i, w> for i < nv in one pass over z, w, V; with
 // norm_slot >= 0 also scal[norm_slot] = ||w||.

@@ -444,7 +444,7 @@ __global__ void build_rhs_kernel(const double* __restrict__ u0, const double* __
 // so that |v| < 2^59: the error is below 2^-55 c times that value.  The steps
 // before v^n are carried as bit patterns and converted in each row's own unit: an
 // integer in the unit of the row before would have lost bits to v^{n-2}.  Values
-// that are not finite or leave the range go through the FP64 row.
+// that are not finite, leave the range or are below 2^-951 go through the FP64 row.
 // Measured at 255^2 x 256: w = L z - s v with 1 and 2 dots 161 us on average
 // (FP64 rows: 287), ||f - L u|| 116 us (300); what bounds them now is the FP64
 // pipe again (2 operations and one a dot), 70 to 80 % busy.
@@ -458,12 +458,14 @@ __global__ void build_rhs_kernel(const double* __restrict__ u0, const double* __
 // multigrid solve), and the other rounding of L moved solutions of the FP32
 // multigrid solves by up to 2e-10.
 constexpr int kFxRows = 4;
+constexpr int kFxTiny = fx::kFxMin + 1081;   // smallest exponent field that fills the least unit
 constexpr int kFxDotVecs = 8;        // vectors a fused launch takes; more go to dots_kernel
 
 struct FxStencil {
   fx::W64 cm;      // c = cm 2^-63 2^ce
   fx::W64 wa[3], wm[3];   // Q1: centre, edge, corner of M + tau K and of M, times 2^(63 - ce)
   int ce;
+  int kc, ke;             // Q1: exponents of 1.5 2^ce over the centre and the edge of M + tau K
   int chunk;       // time steps of a tile
   int xt, yg, planes;   // tiles in x, row groups, planes (3D: m)
   int tiles;
@@ -480,7 +482,37 @@ __device__ __noinline__ double fx_slow_row(const double* __restrict__ vs, long l
                          P == 2 && n > 1 ? vs[q - 2 * g.J] : 0.0);
 }
 
+// Finite differences: which of the lane's rows (mask) are below T (high words of the
+// bit patterns) in all their own values and not zero in all, from memory; `time`:
+// v^n and the steps before it count, not the neighbours.  These rows in FP64.
 template <int KIND, int P>
+__device__ __noinline__ void fx_small_rows(double* y, unsigned mask, int T, bool time, const double* __restrict__ vs,
+                                           long long q, int ix, int iy, int iz, int n, const StencilGeom& g) {
+  auto key = [](double v) { return fx::d_habs(fx::d_bits(v)) | ((unsigned)fx::d_bits(v) != 0); };
+  for (int r = 0; r < kFxRows; ++r) {
+    if (!(mask >> r & 1)) continue;
+    const double* p = vs + q + (long long)r * g.m;
+    const int c = key(p[0]), m1 = g.m - 1;
+    int near = max(c, max(ix > 0 ? key(p[-1]) : 0, ix < m1 ? key(p[1]) : 0));
+    near = max(near, max(iy + r > 0 ? key(p[-g.m]) : 0, iy + r < m1 ? key(p[g.m]) : 0));
+    if constexpr (KIND == kFD3) {
+      const long long m2 = (long long)g.m * g.m;
+      near = max(near, max(iz > 0 ? key(p[-m2]) : 0, iz < m1 ? key(p[m2]) : 0));
+    }
+    const int back = max(n > 0 ? key(p[-g.J]) : 0, P == 2 && n > 1 ? key(p[-2 * g.J]) : 0);
+    if (max(near, back) != 0 && (time ? max(c, back) : near) < T)
+      y[r] = fx_slow_row<KIND, P>(vs, q + (long long)r * g.m, ix, iy + r, iz, n, g);
+  }
+}
+
+// OWN: every row is as accurate as in FP64 for its own values.  Without it a row
+// can hold fewer bits than that where its values are more than 6 bits below the
+// tile's largest: what the solver takes from the rows are norms, dots and Krylov
+// vectors, and in norm the error is below that of FP64 rows.  With OWN, 6 % of the
+// tile's steps of a smooth solution have such rows; all of a solve's passes so cost
+// 5 to 25 % more each (dots at 255^2 x 256 173 us instead of 158, Q1 rows at 127^2 x
+// 64 31 instead of 20), so only bec_apply_A, whose rows a program sees, has it.
+template <int KIND, int P, bool OWN>
 struct FxRow {
   static constexpr int R = kFxRows;
   static constexpr bool D3 = KIND == kFD3, Q1 = KIND == kQ1;
@@ -597,20 +629,37 @@ struct FxRow {
     const int F = max(e - 1081, fx::kFxMin), G = max(F, Fp) + f.ce + 1;
     const int da = min(max(Fp - F, 0), 63), dp = min(max(F - Fp, 0), 63);
     const fx::i64 ra = da > 0 ? 1LL << (da - 1) : 0, rp = dp > 0 ? 1LL << (dp - 1) : 0;
-    const bool plain = em != 0x7FF && fx::fx_normal(G);
+    // else all rows in FP64: not finite, out of range, or too small to fill the unit
+    const bool plain = em != 0x7FF && fx::fx_normal(G) && em >= kFxTiny;
+    int low = 0x7FFFFFFF;                                 // smallest of the rows' larger parts
     q1_rows(w, F, [&](int r, fx::i64 c, fx::i64 eg, fx::i64 d) {
-      const fx::i64 Y = fx::shr(q1_form(f.wa, c, eg, d) + ra, da) - fx::shr(prev[r] + rp, dp);
+      const fx::i64 A = fx::shr(q1_form(f.wa, c, eg, d) + ra, da), M = fx::shr(prev[r] + rp, dp);
       prev[r] = q1_form(f.wm, c, eg, d);
-      if (plain) y[r] = fx::fx_to_d(Y, G);
+      if constexpr (OWN) {
+        const int q = max(high(A), high(M));
+        low = min(low, row_in(r) ? q : 0x7FFFFFFF);
+      }
+      if (plain) y[r] = fx::fx_to_d(A - M, G);
     });
     if (!plain) {
 #pragma unroll
       for (int r = 0; r < R; ++r)
         y[r] = row_in(r) ? fx_slow_row<KIND, P>(vs, q0 + r * m, x, y0 + r, z0, n, g) : 0.0;
+    } else if (OWN && low < 1 << 21) {
+      // An FP64 row's error is about 2^-53 of each of its parts and products, a row's
+      // here about a unit: where none of those looked at reaches 2^53 units, the row
+      // is taken in FP64.
+      const int T = max(F, Fp) + 1076, Tc = min(T + f.kc, 2047) << 20, Te = min(T + f.ke, 2047) << 20;
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        if (row_in(r) && fx::d_habs(w.b[r + 1]) < Tc && max(fx::d_habs(w.b[r]), fx::d_habs(w.b[r + 2])) < Te)
+          y[r] = fx_slow_row<KIND, P>(vs, q0 + r * m, x, y0 + r, z0, n, g);
     }
     ep = e;
     Fp = F;
   }
+  // high word of |v|, less one below zero
+  static __device__ __forceinline__ int high(fx::i64 v) { return (int)(v >> 32) ^ (int)(v >> 63); }
   // y = row values of the slice vs = v^n, whose values are in w
   __device__ __forceinline__ void step(const Raw& w, const double* __restrict__ vs, const StencilGeom& g,
                                        const FxStencil& f, int n, double (&y)[R]) {
@@ -629,7 +678,8 @@ struct FxRow {
     const int G = F + max(s, 0);
     if constexpr (P == 2) ep2 = ep;
     ep = e;
-    if (em == 0x7FF || !fx::fx_normal(G)) {
+    // not finite, out of range, or too small to fill the unit
+    if (em == 0x7FF || !fx::fx_normal(G) || em < kFxTiny) {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         y[r] = row_in(r) ? fx_slow_row<KIND, P>(vs, q0 + r * m, x, y0 + r, z0, n, g) : 0.0;
@@ -637,6 +687,36 @@ struct FxRow {
         prev[r] = (i64)w.b[r + 1];
       }
       return;
+    }
+    // OWN: a row whose own values are all more than 6 bits below the largest holds fewer
+    // than FP64's 53: it is taken in FP64.  The values that count are v^n and its
+    // neighbours, or with c < 1/4, where the error is that of v^n - v^{n-1}, those
+    // two.  Looked at first are a part of them, mostly enough: a lane's own, then the
+    // centres beside it.
+    const int T = (F + 1076) << 20;                       // 2^(F + 53)
+    bool small = false;
+    if constexpr (OWN) {
+      int low = 0x7FFFFFFF;
+      if (s >= 0) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int q = max(max(fx::d_habs(w.b[r]), fx::d_habs(w.b[r + 1])), fx::d_habs(w.b[r + 2]));
+          low = min(low, row_in(r) ? q : 0x7FFFFFFF);
+        }
+      } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          low = min(low, row_in(r) ? max(fx::d_habs(w.b[r + 1]), fx::d_habs((fx::u64)prev[r])) : 0x7FFFFFFF);
+      }
+      small = low < T;
+      if (__any_sync(0xffffffffu, small) && s >= 0) {     // the centres beside the lane's
+        int c = 0x7FFFFFFF;
+#pragma unroll
+        for (int r = 0; r < R; ++r) c = min(c, row_in(r) ? fx::d_habs(w.b[r + 1]) : 0x7FFFFFFF);
+        if (x >= m) c = 0;
+        const int side = max(__shfl_up_sync(0xffffffffu, c, 1), __shfl_down_sync(0xffffffffu, c, 1));
+        small = small && side < T;                        // every lane takes part in the shuffles
+      }
     }
     // shifts round to nearest: a bias of even a small part of a unit, the same at
     // every point, would come back from L^{-1} many times larger
@@ -667,6 +747,14 @@ struct FxRow {
       below = c;
       c = above;
     }
+    if (small) {
+      double t[R];                                        // in memory, y stays in registers
+#pragma unroll
+      for (int r = 0; r < R; ++r) t[r] = y[r];
+      fx_small_rows<KIND, P>(t, in >> 1 & ((1u << R) - 1u), T, s < 0, vs, q0, x, y0, z0, n, g);
+#pragma unroll
+      for (int r = 0; r < R; ++r) y[r] = t[r];
+    }
   }
 };
 
@@ -674,12 +762,12 @@ struct FxRow {
 // stencil_dots_kernel (LAST: vshift is V_{NV-1}); kModeNorms: partials as
 // residual_norms_kernel (aux = f; LAST: without f^2); kModeApply: w = L z (times *sshift if
 // given); kModeResidual: w = aux - L z.
-template <int MODE, int NV, bool LAST, int KIND, int P>
+template <int MODE, int NV, bool LAST, int KIND, int P, bool OWN>
 __global__ void __launch_bounds__(kStencilThreads, NV <= 2 && KIND == kFD ? 3 : 2)
 stencil_fx_kernel(const double* __restrict__ z, const double* __restrict__ aux, double* __restrict__ w,
                   StencilGeom g, FxStencil f, VecList V, const double* __restrict__ vshift,
                   const double* __restrict__ sshift, double* __restrict__ partials) {
-  using Row = FxRow<KIND, P>;
+  using Row = FxRow<KIND, P, OWN>;
   constexpr int R = kFxRows, NA = MODE == kModeDots ? NV + 1 : 2;
   double acc[NA];
 #pragma unroll
@@ -868,6 +956,13 @@ unsigned fx_stencil(const bec_problem* p, const StencilGeom& g, FxStencil& f) {
     f.wm[i] = fx_coef(wm[i], ce);
   }
   f.cm = fx_coef(q1 ? 0.0 : g.c, ce);
+  f.kc = f.ke = 0;
+  if (q1) {
+    std::frexp(1.5 * std::ldexp(1.0, ce) / std::fabs(g.ac), &f.kc);
+    const double ae = std::fabs(g.ae);
+    if (ae > 1e-9 * top) std::frexp(1.5 * std::ldexp(1.0, ce) / ae, &f.ke);
+    else f.ke = 1000;                             // edges never count
+  }
   f.ce = ce;
   f.xt = (p->m + 31) / 32;
   f.yg = (p->m + kFxRows - 1) / kFxRows;
@@ -882,12 +977,12 @@ unsigned fx_stencil(const bec_problem* p, const StencilGeom& g, FxStencil& f) {
   return (unsigned)(blocks < 3 * 152 ? blocks : 3 * 152);
 }
 
-template <int MODE, int NV, bool LAST = false>
+template <int MODE, int NV, bool LAST = false, bool OWN = false>
 void stencil_fx_launch(const bec_problem* p, unsigned grid, const double* z, const double* aux, double* w,
                        const StencilGeom& g, const FxStencil& f, const VecList& L, const double* vshift,
                        const double* sshift) {
 #define BEC_SFX(K, P)                                                                       \
-  stencil_fx_kernel<MODE, NV, LAST, K, P><<<grid, kStencilThreads, 0, p->stream>>>(               \
+  stencil_fx_kernel<MODE, NV, LAST, K, P, OWN><<<grid, kStencilThreads, 0, p->stream>>>(               \
       z, aux, w, g, f, L, vshift, sshift, p->partials)
   if (p->dim == 3) BEC_SFX(kFD3, 1);
   else if (p->desc.space == BEC_SPACE_Q1) BEC_SFX(kQ1, 1);
@@ -909,13 +1004,16 @@ long long stencil_blocks(const bec_problem* p) {
 }
 
 bec_status launch_apply_L(bec_problem* p, const double* v, double* y, double corner,
-                          const double* out_scale) {
+                          const double* out_scale, bool own) {
   const StencilGeom g = geom(p);
   if (corner == 0.0 && fx_rows(p)) {
     FxStencil f;
     const unsigned grid = fx_stencil(p, g, f);
     BEC_LAUNCH_BEGIN(p);
-    stencil_fx_launch<kModeApply, 1>(p, grid, v, nullptr, y, g, f, VecList{}, nullptr, out_scale);
+    if (own)
+      stencil_fx_launch<kModeApply, 1, false, true>(p, grid, v, nullptr, y, g, f, VecList{}, nullptr, out_scale);
+    else
+      stencil_fx_launch<kModeApply, 1>(p, grid, v, nullptr, y, g, f, VecList{}, nullptr, out_scale);
     BEC_LAUNCH_CHECK(p, "apply_L_fx_kernel");
     return BEC_OK;
   }
