@@ -573,26 +573,39 @@ BEC_FX i64 d_to_fx(u64 b, int F) {
   const i64 s = (i64)((int)hi >> 31);
   return (a ^ s) - s;
 }
-// v 2^F rounded to nearest (ties away from zero).  fx_to_d takes |v| >= 2^32
-// with a normal result (fx_normal(F)) itself; the rest goes through ldexp.
-static __host__ __device__ __noinline__ double fx_to_d_slow(i64 v, int F) {
-  return v == 0 ? 0.0 : ldexp((double)v, F);
+// the same for any F: zeros and subnormal numbers as they are
+BEC_FX i64 d_to_fx_sub(u64 b, int F) {
+  const int e = (int)(b >> 52) & 0x7FF;
+  const u64 m = (b & 0xFFFFFFFFFFFFFULL) | (e != 0 ? 1ULL << 52 : 0);
+  const i64 a = (i64)shr_u(m << 10, F + 1085 - (e != 0 ? e : 1));
+  const i64 s = (i64)b >> 63;
+  return (a ^ s) - s;
 }
+// v 2^F rounded to nearest (ties away from zero).  fx_round takes |v| >= 2^32 with
+// a normal result (fx_normal(F)); fx_to_d sends the rest to fx_to_d_slow, which
+// rounds to 53 bits the same way first.
 BEC_FX bool fx_normal(int F) { return F > -1030 && F < 950; }
-BEC_FX double fx_to_d(i64 v, int F) {
-  const i64 s = (i64)((int)(v >> 32) >> 31);
-  const u64 a = (u64)((v ^ s) - s);
-  const unsigned ah = (unsigned)(a >> 32);
-  if (ah == 0) return fx_to_d_slow(v, F);
+BEC_FX double fx_round(u64 a, i64 s, int F) {         // (s ? -a : a) 2^F, s 0 or -1
 #ifdef __CUDA_ARCH__
-  const int lz = __clz((int)ah);
+  const int lz = __clz((int)(a >> 32));
 #else
-  const int lz = __builtin_clz(ah);
+  const int lz = __builtin_clz((unsigned)(a >> 32));
 #endif
   const u64 nrm = a << lz;
   // the 53-bit significand brings the exponent's last unit with it
   const u64 r = ((u64)(unsigned)(F + 1085 - lz) << 52) + (nrm >> 11) + ((nrm >> 10) & 1);
   return bits_d(r | ((u64)s & 0x8000000000000000ULL));
+}
+static __host__ __device__ __noinline__ double fx_to_d_slow(i64 v, int F) {
+  const i64 s = v >> 63;
+  const u64 a = (u64)((v ^ s) - s);
+  return v == 0 ? 0.0 : ldexp(a >> 32 ? fx_round(a, s, 0) : (double)v, F);
+}
+BEC_FX double fx_to_d(i64 v, int F) {
+  const i64 s = (i64)((int)(v >> 32) >> 31);
+  const u64 a = (u64)((v ^ s) - s);
+  if ((unsigned)(a >> 32) == 0) return fx_to_d_slow(v, F);
+  return fx_round(a, s, F);
 }
 
 }  // namespace fx

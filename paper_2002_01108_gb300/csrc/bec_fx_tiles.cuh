@@ -234,15 +234,25 @@ struct DstTile {
       // = ref + 1, stays below 2^62
       constexpr int lg = radix_log(LOGN, 0) + 3;    // R1 5.66 < 2^lg
       c.ref = em - 1022 + lg - 62 - 1;
-      if (c.ref < kFxMin) c.ref = kFxMin;
+      if (c.ref >= kFxMin) {
 #pragma unroll
-      for (int u = 0; u < H; ++u) {
-        r.a[u] = d_to_fx((u64)r.a[u], c.ref);
-        r.a2[u] = d_to_fx((u64)r.a2[u], c.ref);
-        r.b[u] = d_to_fx((u64)r.b[u], c.ref);
-        r.b2[u] = d_to_fx((u64)r.b2[u], c.ref);
-        l += mag(r.a[u]) + mag(r.a2[u]) + mag(r.b[u]) + mag(r.b2[u]);
+        for (int u = 0; u < H; ++u) {
+          r.a[u] = d_to_fx((u64)r.a[u], c.ref);
+          r.a2[u] = d_to_fx((u64)r.a2[u], c.ref);
+          r.b[u] = d_to_fx((u64)r.b[u], c.ref);
+          r.b2[u] = d_to_fx((u64)r.b2[u], c.ref);
+        }
+      } else {                                      // zeros, or next to the subnormal numbers
+#pragma unroll
+        for (int u = 0; u < H; ++u) {
+          r.a[u] = d_to_fx_sub((u64)r.a[u], c.ref);
+          r.a2[u] = d_to_fx_sub((u64)r.a2[u], c.ref);
+          r.b[u] = d_to_fx_sub((u64)r.b[u], c.ref);
+          r.b2[u] = d_to_fx_sub((u64)r.b2[u], c.ref);
+        }
       }
+#pragma unroll
+      for (int u = 0; u < H; ++u) l += mag(r.a[u]) + mag(r.a2[u]) + mag(r.b[u]) + mag(r.b2[u]);
       if (em == 0x7FF) c.ref = kFxNan;
     } else {
       const int mx = max_get<THREADS>(c.mx);
@@ -803,10 +813,14 @@ struct SpecTile : TimeTile<LOGN, LPB> {
   // the line's values as integers below 2^bits; returns their exponent
   static BEC_FX int to_fixed(Ctx& c, Reg& r, int bits) {
     const int em = (int)Join::get(scratch(c), c.s, c.tid, c.L).m;
-    int f = em - 1022 - bits;
-    if (f < kFxMin) f = kFxMin;
+    const int f = em - 1022 - bits;
+    if (f >= kFxMin) {
 #pragma unroll
-    for (int i = 0; i < EPT; ++i) r.v[i] = cx{d_to_fx((u64)r.v[i].x, f), d_to_fx((u64)r.v[i].y, f)};
+      for (int i = 0; i < EPT; ++i) r.v[i] = cx{d_to_fx((u64)r.v[i].x, f), d_to_fx((u64)r.v[i].y, f)};
+    } else {
+#pragma unroll
+      for (int i = 0; i < EPT; ++i) r.v[i] = cx{d_to_fx_sub((u64)r.v[i].x, f), d_to_fx_sub((u64)r.v[i].y, f)};
+    }
     c.f = em == 0x7FF ? kFxNan : 0;
     return f;
   }
