@@ -171,6 +171,10 @@ bec_status bec_batch_solve(bec_batch* b, const double* const* f, double* const* 
     if (opts->left_pc) return batch_einval("BEC_BATCH_PERSISTENT needs right preconditioning");
     for (auto& r : runs) r.ext_pinv = true;
   }
+  auto abandon = [&] {
+    for (auto& r : runs) bec::gmres_run_abandon(r);
+    for (cudaStream_t s : b->streams) (void)cudaStreamSynchronize(s);
+  };
   bec_status first_error = BEC_OK;
   std::vector<char> busy(b->streams.size());
   std::vector<int> at_iter;
@@ -226,7 +230,10 @@ bec_status bec_batch_solve(bec_batch* b, const double* const* f, double* const* 
           int* ctr = b->ctr_dev + (size_t)launches * kCtrInts;
           const bec_status st = bec::persist_launch(jh, b->jobs_dev + slot, nj, &q, ctr,
                                                     bec::persist_take_withhold(), b->streams[si]);
-          if (st != BEC_OK) return st;
+          if (st != BEC_OK) {
+            abandon();
+            return st;
+          }
           ++b->persist_launches;
           // the launch's error word, read once the round has drained
           BEC_CUDA_TRY(cudaMemcpyAsync(b->err_host + launches, ctr + 1, sizeof(int),
@@ -255,6 +262,7 @@ bec_status bec_batch_solve(bec_batch* b, const double* const* f, double* const* 
       }
     for (int c = 0; c < launches; ++c)
       if (b->err_host[c] != 0) {
+        abandon();
         bec::set_error("persistent batch launch: a bounded wait for an earlier pass ran out");
         return BEC_ETIMEOUT;
       }

@@ -172,12 +172,7 @@ bec_status enqueue_iteration(GmresRun& r) {
   return BEC_OK;
 }
 
-}  // namespace
-
-// Advance one step.  `enqueued` tells the caller that work ending in a
-// scalar read was put on the stream and the next call must come after the
-// stream has drained.
-bec_status gmres_run_step(GmresRun& r, bool* enqueued) {
+bec_status run_step(GmresRun& r, bool* enqueued) {
   bec_problem* p = r.p;
   *enqueued = false;
   switch (r.state) {
@@ -317,6 +312,21 @@ bec_status gmres_run_step(GmresRun& r, bool* enqueued) {
       return r.status;
   }
   return BEC_OK;
+}
+
+}  // namespace
+
+// Advance one step.  `enqueued` tells the caller that work ending in a
+// scalar read was put on the stream and the next call must come after the
+// stream has drained.
+bec_status gmres_run_step(GmresRun& r, bool* enqueued) {
+  const bec_status s = run_step(r, enqueued);
+  if (s != BEC_OK) gmres_run_abandon(r);
+  return s;
+}
+
+void gmres_run_abandon(GmresRun& r) {
+  if (!r.x_nonzero && r.state != GmresRun::DONE) (void)launch_zero(r.p, r.u);
 }
 
 void gmres_run_pinv_operands(const GmresRun& r, const double** y, double** z,

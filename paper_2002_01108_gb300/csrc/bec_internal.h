@@ -207,6 +207,9 @@ struct GmresRun {
 void gmres_run_init(GmresRun& r, bec_problem* p, const double* f, double* u,
                     const bec_gmres_opts& o, bool use_graphs);
 bec_status gmres_run_step(GmresRun& r, bool* enqueued);
+// u = 0 for a run that ends early, unless an update or a first guess is in it (the
+// first update writes u)
+void gmres_run_abandon(GmresRun& r);
 // Operands of the P_eps^{-1} of the coming Arnoldi step (state ITER, right
 // preconditioning): z = P^{-1} (s y) with s = *scale_dev.
 void gmres_run_pinv_operands(const GmresRun& r, const double** y, double** z,
