@@ -7,8 +7,11 @@
 // addition costs 1/30 of an FP64 addition and a 64-bit product by a constant
 // (three 32-bit products) about 1/9 of an FP64 product.  The transforms are
 // bounded linear maps of one line at a time, so a common exponent per line
-// pair is enough: with the values as 62-bit integers the rounding
-// errors are below those of the FP64 transform (whose values carry 53 bits).
+// pair is enough: the values are 62-bit integers, where FP64 carries 53 bits of
+// each.  Measured for P_eps^{-1} against extended precision (2-norm, 63 cases: 1D to
+// 3D, N = 64 to 1024, eps = 1e-3 to 1, a = 1e-5 to 1; flat, alternating and smooth
+// data): from 0.01 to 1.2 times the error of the floating-point passes, below it
+// in most cases.
 //
 // Representation.  A line pair (two real lines a, b packed as a + i b) holds
 // 64-bit integers v with one exponent F: the value is v 2^F.

@@ -27,7 +27,6 @@ constexpr int S_REF = 0, S_BETA = 1, S_W = 2, S_RES = 3, S_TRUE = 4, S_WB = 6, S
 
 }  // namespace
 
-// z = P_eps^{-1} (s y), s = *scale_dev (1 if null)
 double pinv_scale(const bec_problem* p) {
   const double n = (double)(p->m + 1);
   const double per_axis = (2.0 / n) / 16.0;   // (orthonormal / raw)^2 for one forward+inverse pair
@@ -36,6 +35,7 @@ double pinv_scale(const bec_problem* p) {
   return scale;
 }
 
+// z = P_eps^{-1} (s y), s = *scale_dev (1 if null)
 bec_status apply_pinv(bec_problem* p, const double* y, double* z, const double* scale_dev) {
   NvtxRange range("bec P_eps^-1");
   const int fp64 = p->desc.precision == BEC_PC_FP64;

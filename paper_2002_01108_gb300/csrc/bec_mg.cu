@@ -740,8 +740,8 @@ ilu_sweep_async_kernel(v2_t<T>* __restrict__ x, v2_t<T>* work, const v2_t<T>* ri
 // block barrier every D steps enough, and reads that row from a ring in shared
 // memory.  The operands are staged by cp.async D - 1 steps ahead, in slots of
 // the lane's own; a step reads the next one's and forms its coefficients while
-// the recurrence of this one is in flight.  The arithmetic is the wavefront
-// kernel's, operation by operation.  The backward sweep is the forward one on
+// the recurrence of this one is in flight.  The sums run in the wavefront kernel's
+// order (the results differ by FP32 roundings).  The backward sweep is the forward one on
 // the mirrored grid.
 //
 // The forward result goes to a buffer of its own in wavefront order: 32 lanes

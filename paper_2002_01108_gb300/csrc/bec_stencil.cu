@@ -445,9 +445,10 @@ __global__ void build_rhs_kernel(const double* __restrict__ u0, const double* __
 // before v^n are carried as bit patterns and converted in each row's own unit: an
 // integer in the unit of the row before would have lost bits to v^{n-2}.  Values
 // that are not finite, leave the range or are below 2^-951 go through the FP64 row.
-// Measured at 255^2 x 256: w = L z - s v with 1 and 2 dots 161 us on average
-// (FP64 rows: 287), ||f - L u|| 116 us (300); what bounds them now is the FP64
-// pipe again (2 operations and one a dot), 70 to 80 % busy.
+// Measured at 255^2 x 256: w = L z - s v with 1 and 2 dots 158 us on average
+// (FP64 rows: 287), ||f - L u|| 127 us (300); what bounds them now is the FP64
+// pipe again (2 operations and one a dot), 70 to 80 % busy.  Converting v^{n-1}
+// again only where the unit changes costs more branches than it saves (183 us).
 //
 // Q1 rows take six products, three of them by M, which the next step's row
 // subtracts: a lane keeps M v^{n-1} instead of the values.  At 127^2 x 64 (1M
@@ -942,7 +943,11 @@ fx::W64 fx_coef(double v, int ce) {
   return fx::split64(w);
 }
 
-// blocks: what the card holds at once (3 a SM), or fewer
+// Blocks of a launch, or fewer: 3 an SM.  The finite-difference kernels with up to
+// 2 vectors are held to the registers for that (80 a thread, up to 120 bytes of
+// them in local memory); the others take 118 to 128 and run 2 at a time, so that the
+// last third of their blocks follows the first two.
+constexpr int kFxBlocks = 3 * 152;
 unsigned fx_stencil(const bec_problem* p, const StencilGeom& g, FxStencil& f) {
   int ce;
   const bool q1 = p->desc.space == BEC_SPACE_Q1;
@@ -968,13 +973,13 @@ unsigned fx_stencil(const bec_problem* p, const StencilGeom& g, FxStencil& f) {
   f.yg = (p->m + kFxRows - 1) / kFxRows;
   f.planes = p->dim == 3 ? p->m : 1;
   const int per = f.xt * f.yg * f.planes;          // at most 2^23
-  const long long warps = 3LL * 152 * (kStencilThreads / 32);
-  // the longest chunk that still gives every warp of the card a tile
+  const long long warps = (long long)kFxBlocks * (kStencilThreads / 32);
+  // the longest chunk that still gives every warp of the launch a tile
   f.chunk = 16;
   while (f.chunk > 1 && (long long)per * ((p->N + f.chunk - 1) / f.chunk) < warps) f.chunk /= 2;
   f.tiles = per * ((p->N + f.chunk - 1) / f.chunk);
   const int blocks = (f.tiles + kStencilThreads / 32 - 1) / (kStencilThreads / 32);
-  return (unsigned)(blocks < 3 * 152 ? blocks : 3 * 152);
+  return (unsigned)std::min(blocks, kFxBlocks);
 }
 
 template <int MODE, int NV, bool LAST = false, bool OWN = false>
@@ -1058,22 +1063,22 @@ bec_status launch_stencil_dots(bec_problem* p, const double* z, double* w,
     }
     BEC_LAUNCH_CHECK(p, "stencil_dots_fx_kernel");
   } else {
-  BEC_LAUNCH_BEGIN(p);
-  switch (n) {
+    BEC_LAUNCH_BEGIN(p);
+    switch (n) {
 #define BEC_SD_CASE(NV)                                                                  \
-  case NV:                                                                               \
-    stencil_dots_launch<NV>(var, p->stream, z, w, g, L, vshift, sshift, p->partials);   \
-    break;
-    BEC_SD_CASE(1) BEC_SD_CASE(2) BEC_SD_CASE(3) BEC_SD_CASE(4) BEC_SD_CASE(5) BEC_SD_CASE(6)
-    BEC_SD_CASE(7) BEC_SD_CASE(8) BEC_SD_CASE(9) BEC_SD_CASE(10) BEC_SD_CASE(11) BEC_SD_CASE(12)
-    BEC_SD_CASE(13) BEC_SD_CASE(14) BEC_SD_CASE(15) BEC_SD_CASE(16) BEC_SD_CASE(17)
-    BEC_SD_CASE(18) BEC_SD_CASE(19) BEC_SD_CASE(20) BEC_SD_CASE(21) BEC_SD_CASE(22)
-    BEC_SD_CASE(23) BEC_SD_CASE(24) BEC_SD_CASE(25) BEC_SD_CASE(26) BEC_SD_CASE(27)
-    BEC_SD_CASE(28) BEC_SD_CASE(29) BEC_SD_CASE(30) BEC_SD_CASE(31) BEC_SD_CASE(32)
+    case NV:                                                                               \
+      stencil_dots_launch<NV>(var, p->stream, z, w, g, L, vshift, sshift, p->partials);   \
+      break;
+      BEC_SD_CASE(1) BEC_SD_CASE(2) BEC_SD_CASE(3) BEC_SD_CASE(4) BEC_SD_CASE(5) BEC_SD_CASE(6)
+      BEC_SD_CASE(7) BEC_SD_CASE(8) BEC_SD_CASE(9) BEC_SD_CASE(10) BEC_SD_CASE(11) BEC_SD_CASE(12)
+      BEC_SD_CASE(13) BEC_SD_CASE(14) BEC_SD_CASE(15) BEC_SD_CASE(16) BEC_SD_CASE(17)
+      BEC_SD_CASE(18) BEC_SD_CASE(19) BEC_SD_CASE(20) BEC_SD_CASE(21) BEC_SD_CASE(22)
+      BEC_SD_CASE(23) BEC_SD_CASE(24) BEC_SD_CASE(25) BEC_SD_CASE(26) BEC_SD_CASE(27)
+      BEC_SD_CASE(28) BEC_SD_CASE(29) BEC_SD_CASE(30) BEC_SD_CASE(31) BEC_SD_CASE(32)
 #undef BEC_SD_CASE
-    default: return BEC_EINVAL;
-  }
-  BEC_LAUNCH_CHECK(p, "stencil_dots_kernel");
+      default: return BEC_EINVAL;
+    }
+    BEC_LAUNCH_CHECK(p, "stencil_dots_kernel");
   }
   const bec_status s = launch_finish_dots(p, n, nb, sigma, hout, nullptr, norm_slot);
   if (s != BEC_OK || nv <= most) return s;
@@ -1116,12 +1121,12 @@ bec_status launch_residual_norms(bec_problem* p, const double* f, const double* 
       stencil_fx_launch<kModeNorms, 1>(p, gx, u, f, nullptr, g, x, VecList{}, nullptr, nullptr);
     BEC_LAUNCH_CHECK(p, "residual_norms_fx_kernel");
   } else {
-  BEC_LAUNCH_BEGIN(p);
+    BEC_LAUNCH_BEGIN(p);
 #define BEC_RN_LAUNCH(K, P) \
-  residual_norms_kernel<K, P><<<grid, kStencilThreads, 0, p->stream>>>(f, u, p->partials, g)
-  BEC_STENCIL_SWITCH(variant_of(p), BEC_RN_LAUNCH)
+    residual_norms_kernel<K, P><<<grid, kStencilThreads, 0, p->stream>>>(f, u, p->partials, g)
+    BEC_STENCIL_SWITCH(variant_of(p), BEC_RN_LAUNCH)
 #undef BEC_RN_LAUNCH
-  BEC_LAUNCH_CHECK(p, "residual_norms_kernel");
+    BEC_LAUNCH_CHECK(p, "residual_norms_kernel");
   }
   BEC_LAUNCH_BEGIN(p);
   finish_norms_kernel<<<1, 256, 0, p->stream>>>(p->partials, nblk, p->scal, slot, fslot,
