@@ -110,31 +110,40 @@ def net_fwd_flops(m: int) -> float:
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, from one ncu capture
 # of each kernel at this workload (the P_eps^-1 passes of the second of three
-# applies of `bench.py --ncu-case pinv_fp32`; the command is in the committed
-# DRAM-traffic summary under profiles/).  Each entry carries a SHA-256 prefix
-# of the CUDA sources the kernel is built from, taken when the counters were
-# read: if those sources have changed since, the figure no longer describes
-# the kernel and the bench reports null.  The writes are what left L2 while
-# the kernel ran.
+# applies of `bench.py --ncu-case pinv_fp64` and `pinv_fp32`; the commands are
+# in the committed DRAM-traffic summary under profiles/).  Each entry carries a
+# SHA-256 prefix of the CUDA sources the kernel is built from, taken when the
+# counters were read: if those sources have changed since, the figure no longer
+# describes the kernel and the bench reports null.  The writes are what left L2
+# while the kernel ran.
 KERNEL_SOURCES = {
     "dst_rows_kernel": ("bec_dst.cu", "bec_passes.cuh", "bec_fft.cuh"),
     "dst_cols_kernel": ("bec_dst.cu", "bec_passes.cuh", "bec_fft.cuh"),
     "time_pass_kernel": ("bec_time.cu", "bec_passes.cuh", "bec_fft.cuh"),
     "dst_cols16_tma_kernel": ("bec_dst.cu", "bec_passes.cuh", "bec_fft.cuh", "bec_tma.cuh"),
     "time_pass16_tma_kernel": ("bec_time.cu", "bec_passes.cuh", "bec_fft.cuh", "bec_tma.cuh"),
+    "dst_rows_fx_kernel": ("bec_fx_dst.cu", "bec_fx_tiles.cuh", "bec_fx.cuh"),
+    "dst_cols_fx_kernel": ("bec_fx_dst.cu", "bec_fx_tiles.cuh", "bec_fx.cuh"),
+    "time_fx_kernel": ("bec_fx_time.cu", "bec_fx_tiles.cuh", "bec_fx.cuh"),
 }
 NCU_TRAFFIC = {
-    ("dst_rows_kernel", "fp32"): (133208320 + 34398464, "d8db73df32f0a703"),
-    ("dst_cols16_tma_kernel", "fp32"): (66874624 + 4049920, "99e057cadaa803e3"),
-    ("time_pass16_tma_kernel", "fp32"): (66894336 + 4122880, "dac5a038203bb35d"),
+    ("dst_rows_fx_kernel", "fp64"): (133265408 + 80480256, "732749b164245d01"),
+    ("dst_cols_fx_kernel", "fp64"): (133276672 + 83912448, "732749b164245d01"),
+    ("time_fx_kernel", "fp64"): (269834240 + 87781888, "86e30705781e60f0"),
+    ("dst_rows_kernel", "fp32"): (133201408 + 34096640, "d8db73df32f0a703"),
+    ("dst_cols16_tma_kernel", "fp32"): (66873344 + 3761152, "99e057cadaa803e3"),
+    ("time_pass16_tma_kernel", "fp32"): (66887424 + 4157952, "4a0194dc2c727b19"),
 }
 # DRAM bytes of one whole P_eps^-1 apply (the five passes of the same
 # capture) and the kernels whose sources they were taken on
 NCU_PINV_BYTES = {
-    "fp32": ((133208320 + 34398464) + (66874624 + 4049920) + (66894336 + 4122880)
-             + (66874880 + 3893248) + (66878720 + 69490944),
+    "fp64": ((133265408 + 80480256) + (133276672 + 83912448) + (269834240 + 87781888)
+             + (133269248 + 83793408) + (133310464 + 70642944),
+             {"dst_rows_fx_kernel": "732749b164245d01", "time_fx_kernel": "86e30705781e60f0"}),
+    "fp32": ((133201408 + 34096640) + (66873344 + 3761152) + (66887424 + 4157952)
+             + (66874624 + 3750400) + (66878464 + 69615360),
              {"dst_rows_kernel": "d8db73df32f0a703", "dst_cols16_tma_kernel": "99e057cadaa803e3",
-              "time_pass16_tma_kernel": "dac5a038203bb35d"}),
+              "time_pass16_tma_kernel": "4a0194dc2c727b19"}),
 }
 
 
@@ -578,7 +587,7 @@ def roofline(form, kernels, U, iters=2):
     roof["avg_launch_ms"] = avg_ms
     roof["traffic"] = ncu_traffic(dom, form)
     roof["traffic_source"] = ("dram__bytes_read.sum + dram__bytes_write.sum of one launch, ncu capture "
-                              "of bench.py --ncu-case pinv_fp32 on the kernel's current sources"
+                              f"of bench.py --ncu-case pinv_{form} on the kernel's current sources"
                               if roof["traffic"] is not None else
                               "no ncu capture of the kernel's current sources")
     return roof

@@ -4,7 +4,7 @@
 // three radix passes through shared memory.  What bounds a pass: about 100
 // integer instructions an element at 16 warps an SM (128 registers a thread),
 // next to 16 bytes an element of HBM traffic.  Measured at 255^2 x 256 (16.6M
-// unknowns): y-DST 92 us, x-DST 105 us, where the floating-point passes take
+// unknowns): y-DST 93 us, x-DST 105 us, where the floating-point passes take
 // 550 us (17 FP64 instructions an element at 2 a clock and SM).
 #include <cuda_runtime.h>
 

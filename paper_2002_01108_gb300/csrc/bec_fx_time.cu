@@ -4,7 +4,8 @@
 // The division by lambda'_k + tau mu is a product by a table of reciprocals in
 // fixed point (16 bytes a mode and frequency, 8 bytes an unknown read from
 // HBM); computing them would take FP64 operations.  Measured at 255^2 x 256:
-// 189 us, where the floating-point pass takes 1042 us.
+// 200 us, where the floating-point pass takes 1042 us (187 us with one exponent for
+// all frequencies of a tile, which lost up to 22 bits of the factors).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -228,7 +229,7 @@ void fx_free(bec_problem* p) {
 }
 
 // Lengths from 32: there the whole apply is faster at every size measured, from
-// 37 against 65 us at 63 x 64 (1D) to 1.14 against 6.87 ms at 255^2 x 512;
+// 44 against 71 us at 63 x 64 (1D) to 1.19 against 6.86 ms at 255^2 x 512;
 // shorter transforms would leave a block less than a warp.
 bool fx_wanted(const bec_problem_desc* d, int logn, int logt) {
   return d->precision == BEC_PC_FP64 && d->route == BEC_ROUTE_FST && logn >= 5 && logt >= 5;
@@ -240,8 +241,8 @@ bec_status fx_setup(bec_problem* p) {
   // 16 line pairs a block (256-byte segments across the lines); 8 for the long
   // lines whose blocks would otherwise pass 512 threads, and where both passes
   // still have 64 threads a block with 8: more and smaller blocks overlap
-  // better there (255^2 x 256: 581 against 614 us an apply), while shorter
-  // lines lose (63^3 x 64: 733 against 671 us)
+  // better there (255^2 x 256: 596 against 621 us an apply), while shorter
+  // lines lose (63^3 x 64: 743 against 682 us)
   t.lpb = p->tab.space.logn >= 9 || p->tab.time.logn >= 9 || (p->tab.space.logn == 8 && p->tab.time.logn >= 7)
               ? 8 : 16;
   // one exponent a tile: of rows, and of columns or modes
